@@ -7,6 +7,7 @@
 
 #include "wrs_device.cuh"
 #include "wrs_fov.cuh"
+#include "wrs_staged.cuh"
 
 namespace wrs {
 
@@ -62,8 +63,8 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // Waits for phase `parity` of `bar` to complete; false once limit_ns has passed.
-static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
+// The call that finds the phase complete (the common one) stays inline.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
   const uint64_t t0 = global_ns();
   for (;;) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -71,29 +72,8 @@ static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t pa
   }
 }
 
-// Byte offsets of one stage's planes in shared memory (tile of T pixels).
-// cs = 2 (FP16 colour: K planes of the weights' low 16 bits, then K planes of
-// 8-byte records {r, g, b, w_hi}) or 4 (FP32 colour: K float4 {w, r, g, b}
-// record planes, starting at `col`; `wt` == `col`).
-struct StageLayout {
-  uint32_t frame, W, P, key, wt, col, bytes;
-};
-
-__host__ __device__ __forceinline__ StageLayout stage_layout(int T, int K, int cs, bool resolve) {
-  StageLayout L;
-  L.frame = 0;
-  L.W = 12u * T;
-  L.P = L.W + 4u * T;
-  L.key = L.P + 4u * T;
-  if (cs == 2) {
-    L.wt = L.key + 4u * K * T;
-    L.col = L.wt + (resolve ? 2u * K * T : 0u);
-    L.bytes = L.col + (resolve ? 8u * K * T : 0u);
-  } else {
-    L.wt = L.col = L.key + 4u * K * T;
-    L.bytes = L.col + (resolve ? 16u * K * T : 0u);
-  }
-  return L;
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
+  return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, limit_ns);
 }
 
 // Warp-wide: lane 0 arms `bar` for the tile's bytes (plus extra_tx, which is
@@ -185,74 +165,56 @@ __device__ __forceinline__ void draw_tile_uniforms_warp(const StreamDev& s, cons
   }
 }
 
-// Computes consumer thread `tid`'s PX pixels of a landed tile from shared
-// memory; returns how many of them replaced a slot. LIT: the literal n = 1
-// rule (KT = 1).
-template <int KT, bool F16, int PX, int T, bool LIT = false, int KM = FoldCap<KT>::value>
-__device__ __forceinline__ int compute_tile(const StreamDev& s, const FrameDev& f,
-                                            const StageLayout& L, const uint8_t* st,
-                                            const float* u, int64_t p0, float d_f, int tid,
-                                            const FoldIn<KM>* pre = nullptr) {
-  const int tl = tid * PX;
-  const int64_t p = p0 + tl;
-  if (p >= s.hw) return 0;
-  Src src;
-  src.W = reinterpret_cast<const float*>(st + L.W);
-  src.P = reinterpret_cast<const float*>(st + L.P);
-  src.key = reinterpret_cast<const float*>(st + L.key);
-  src.wt = reinterpret_cast<const uint16_t*>(st + L.wt);
-  src.col = st + L.col;
-  src.stride = T;
-  src.at = tl;
-  src.frame = reinterpret_cast<const float*>(st + L.frame) + 3 * tl;
-  src.u = u + tl;
-  if constexpr (LIT) {
-    if (f.fov != nullptr) return push_group_literal<F16, PX, true, true>(s, f, static_cast<int>(p), src, d_f);
-    return push_group_literal<F16, PX, true, false>(s, f, static_cast<int>(p), src, d_f);
-  } else {
-    if (f.fov != nullptr) return push_group<KT, F16, PX, true, true, KM>(s, f, static_cast<int>(p), src, d_f, pre);
-    return push_group<KT, F16, PX, true, false, KM>(s, f, static_cast<int>(p), src, d_f, pre);
+// What a consumer thread of a tile knows before the tile has landed: its first
+// pixel p = (x, y) (no pixel if p >= hw), the flush bits of its PX pixels and,
+// in the band this frame folds, the fold's inputs. Loaded ahead of the wait,
+// so that their latency passes while the tile is still in flight.
+template <int KM>
+struct TilePx {
+  uint32_t p, flush;
+  int x, y;
+  bool folding;
+  FoldIn<KM> fold;
+};
+
+// Fills t for the pixels at t.p (t.x and t.y already set).
+template <int KM, int PX, bool FOLD>
+__device__ __forceinline__ void tile_ahead(const StreamDev& s, const FrameDev& f, TilePx<KM>& t) {
+  t.flush = 0;
+  t.folding = false;
+  if (t.p >= static_cast<uint32_t>(s.hw)) return;
+  t.flush = flush_bits<PX>(f, t.p);
+  if constexpr (FOLD && PX == 1) {
+    if (s.K > 2 && s.K <= KM && folds_now(f, t.p)) {
+      fold_load(s, s.idx, s.K, f.t, t.p, t.fold);
+      t.folding = true;
+    }
   }
 }
 
-// Before a consumer waits for its tile: if the tile's pixel of thread `tid`
-// (one pixel per thread) is in the band this frame folds, load the fold's
-// inputs now, so that their latency passes while the tile is still in flight.
-// Returns whether `in` was filled.
-template <int KM, int PX>
-__device__ __forceinline__ bool prefetch_fold(const StreamDev& s, const FrameDev& f, int64_t p0,
-                                              int tid, FoldIn<KM>& in) {
-  if constexpr (PX == 1) {
-    const int64_t p = p0 + tid;
-    if (s.K > 2 && s.K <= KM && p < s.hw && folds_now(f, p)) {
-      fold_load(s, s.idx, s.K, f.t, p, in);
-      return true;
-    }
+// Computes consumer thread `tid`'s PX pixels of a landed tile from shared
+// memory; returns how many of them replaced a slot. LIT: the literal n = 1
+// rule (KT = 1). FILTER >= 0: the thread first foveates its pixels of the
+// frame from `fv` into the stage's frame segment (the producer copied no
+// frame); each thread writes and then reads only its own pixels there.
+template <int KT, bool F16, int PX, int T, bool LIT, int FILTER, int KM>
+__device__ __forceinline__ int compute_tile(const StreamDev& s, const FrameDev& f, const FovDev& fv,
+                                            uint8_t* st, const float* u, const TilePx<KM>& t,
+                                            float d_f, int tid) {
+  if (t.p >= static_cast<uint32_t>(s.hw)) return 0;
+  if constexpr (FILTER >= 0) {
+    float* fr = reinterpret_cast<float*>(st) + 3 * tid * PX;
+#pragma unroll
+    for (int i = 0; i < PX; ++i) fov_pixel<FILTER>(fv, f.gx, f.gy, t.x + i, t.y, fr + 3 * i);
   }
-  return false;
+  if constexpr (LIT)
+    return push_staged_literal<F16, PX, T>(s, f, st, u, t.p, t.x, t.y, d_f, tid, t.flush);
+  else
+    return push_staged<KT, F16, PX, T, KM>(s, f, st, u, t.p, t.x, t.y, d_f, tid, t.flush,
+                                           t.folding ? &t.fold : nullptr);
 }
 
 // Adds a warp's counts to a running total: one atomic per warp.
-// As compute_tile, with the thread's PX pixels of the frame foveated from
-// `fv` into the stage's frame segment first (the producer copied no frame);
-// each thread writes and then reads only its own pixels there.
-template <int KT, bool F16, int PX, int T, bool LIT, int FILTER, int KM = FoldCap<KT>::value>
-__device__ __forceinline__ int compute_tile_fov(const StreamDev& s, const FrameDev& f,
-                                                const FovDev& fv, const StageLayout& L,
-                                                uint8_t* st, const float* u, int64_t p0,
-                                                float d_f, int tid,
-                                                const FoldIn<KM>* pre = nullptr) {
-  const int tl = tid * PX;
-  const int64_t p = p0 + tl;
-  if (p >= s.hw) return 0;
-  int y, x;
-  row_col(s, static_cast<int>(p), y, x);
-  float* fr = reinterpret_cast<float*>(st + L.frame) + 3 * tl;
-#pragma unroll
-  for (int i = 0; i < PX; ++i) fov_pixel<FILTER>(fv, f.gx, f.gy, x + i, y, fr + 3 * i);
-  return compute_tile<KT, F16, PX, T, LIT, KM>(s, f, L, st, u, p0, d_f, tid, pre);
-}
-
 __device__ __forceinline__ void add_warp_count(unsigned long long* total, int count, int lane) {
   const unsigned c = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(count));
   if (lane == 0 && c != 0) atomicAdd(total, static_cast<unsigned long long>(c));
@@ -318,15 +280,19 @@ __device__ __forceinline__ bool flag_raised(const Ring& r) {
 template <typename TileFn>
 __device__ __forceinline__ int produce(const Ring& r, int my_tiles, uint64_t timeout_ns, int lane,
                                        TileFn tile_fn) {
-  int it = 0;
+  int it = 0, stg = 0;
+  uint32_t phase = 1;  // of the stage's last release; the first S tiles wait for none
   for (; it < my_tiles; ++it) {
-    const int stg = it % r.S;
-    if (it >= r.S && !mbar_wait_bounded(&r.empty[stg], ((it / r.S) - 1) & 1u, timeout_ns)) {
+    if (it >= r.S && !mbar_wait_bounded(&r.empty[stg], phase, timeout_ns)) {
       raise_flag(r);
       break;
     }
     if (flag_raised(r)) break;
     tile_fn(it, r.stage(stg), r.u(stg), &r.full[stg], lane);
+    if (++stg == r.S) {
+      stg = 0;
+      phase ^= 1u;
+    }
   }
   return it;
 }
@@ -337,16 +303,22 @@ __device__ __forceinline__ int produce(const Ring& r, int my_tiles, uint64_t tim
 template <typename BeforeFn, typename ComputeFn>
 __device__ __forceinline__ void consume(const Ring& r, int my_tiles, uint64_t timeout_ns, int lane,
                                         BeforeFn before_fn, ComputeFn compute_fn) {
+  int stg = 0;
+  uint32_t phase = 0;
   for (int it = 0; it < my_tiles; ++it) {
-    const int stg = it % r.S;
     before_fn(it);
-    if (!mbar_wait_bounded(&r.full[stg], (it / r.S) & 1u, timeout_ns)) {
+    if (!mbar_wait_bounded(&r.full[stg], phase, timeout_ns)) {
       raise_flag(r);
       break;
     }
     compute_fn(it, r.stage(stg), r.u(stg));
+    fence_stage_writes();
     __syncwarp();
     if (lane == 0) mbar_arrive(&r.empty[stg]);
+    if (++stg == r.S) {
+      stg = 0;
+      phase ^= 1u;
+    }
   }
 }
 

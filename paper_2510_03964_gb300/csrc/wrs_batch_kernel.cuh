@@ -77,25 +77,13 @@ __device__ __forceinline__ void flush_count(unsigned long long* replaced_s, int 
 constexpr int kFamF16K48 = 0, kFamF32K48 = 1, kFamAll = 2;
 
 // One tile of entry e: the update from the staged frame, or (FOVF >= 0) from
-// the frame foveated on read.
-// pre: the fold inputs loaded before the wait (for up to 8 slots, used as
-// they are: no narrowed copy, which would have to live in local memory), or
-// null. The generic-K and literal forms take none.
+// the frame foveated on read. The fold inputs are held for up to 8 slots
+// whatever the stream's K (no narrowed copy, which would have to live in local
+// memory); the generic-K and literal forms load their own.
 template <int KT, bool F16, int PX, int T, bool LIT, int FOVF>
-__device__ __forceinline__ int tile(const BatchEntry& e, const StageLayout& L, uint8_t* st,
-                                    const float* u, int64_t p0, float d_f, int tid,
-                                    const wrs::FoldIn<8>* pre = nullptr) {
-  if constexpr (KT == 4 || KT == 8) {
-    if constexpr (FOVF >= 0)
-      return wrs::compute_tile_fov<KT, F16, PX, T, LIT, FOVF, 8>(e.s, e.f, e.fv, L, st, u, p0, d_f, tid, pre);
-    else
-      return wrs::compute_tile<KT, F16, PX, T, LIT, 8>(e.s, e.f, L, st, u, p0, d_f, tid, pre);
-  } else {
-    if constexpr (FOVF >= 0)
-      return wrs::compute_tile_fov<KT, F16, PX, T, LIT, FOVF>(e.s, e.f, e.fv, L, st, u, p0, d_f, tid);
-    else
-      return wrs::compute_tile<KT, F16, PX, T, LIT>(e.s, e.f, L, st, u, p0, d_f, tid);
-  }
+__device__ __forceinline__ int tile(const BatchEntry& e, uint8_t* st, const float* u,
+                                    const wrs::TilePx<8>& px, float d_f, int tid) {
+  return wrs::compute_tile<KT, F16, PX, T, LIT, FOVF>(e.s, e.f, e.fv, st, u, px, d_f, tid);
 }
 
 // The producer's work for one tile of entry e: its uniforms, then its bulk
@@ -164,10 +152,7 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
                             }
                           });
   } else {
-    // fold inputs of entries that compute with K = 4 or 8, loaded before the
-    // wait; the generic-K arithmetic loads its own (the literal rule has none)
-    wrs::FoldIn<8> fin;
-    bool folding = false;
+    wrs::TilePx<8> px;
     int ei = 0;        // entry of the consumer's current tile
     int replaced = 0;  // this thread's replacements in entry ei so far
     wrs::consume(r, my_tiles, a.timeout_ns, lane, [&](int it) {
@@ -178,35 +163,35 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
         ei = next;
       }
       const BatchEntry& e = a.e[ei];
-      const int64_t p0 = static_cast<int64_t>(g - e.tile0) * T;
-      folding = e.code < 4 && wrs::prefetch_fold<8, PX>(e.s, e.f, p0, tid, fin);
-    }, [&](int it, uint8_t* st, const float* u) {
-      const int g = first + it * step;
+      px.p = static_cast<uint32_t>(g - e.tile0) * T + tid * PX;
+      wrs::row_col(e.s, static_cast<int>(px.p), px.y, px.x);
+      // fold inputs only for entries that compute with K = 4 or 8
+      if (e.code < 4) {
+        wrs::tile_ahead<8, PX, true>(e.s, e.f, px);
+      } else {
+        wrs::tile_ahead<8, PX, false>(e.s, e.f, px);
+      }
+    }, [&](int, uint8_t* st, const float* u) {
       const BatchEntry& e = a.e[ei];
-      const int64_t p0 = static_cast<int64_t>(g - e.tile0) * T;
-      const bool resolve = stage_records(e);
       const float d_f = d_f_s[ei];
       if (failed_s[ei] != 0) return;
-      const wrs::FoldIn<8>* pre = folding ? &fin : nullptr;
       int rc;
       if constexpr (FAM == kFamF16K48) {
-        rc = e.code == 0
-                 ? tile<4, true, PX, T, false, FOVF>(e, wrs::stage_layout(T, 4, 2, resolve), st, u, p0, d_f, tid, pre)
-                 : tile<8, true, PX, T, false, FOVF>(e, wrs::stage_layout(T, 8, 2, resolve), st, u, p0, d_f, tid, pre);
+        rc = e.code == 0 ? tile<4, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid)
+                         : tile<8, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid);
       } else if constexpr (FAM == kFamF32K48) {
-        rc = e.code == 2
-                 ? tile<4, false, PX, T, false, FOVF>(e, wrs::stage_layout(T, 4, 4, resolve), st, u, p0, d_f, tid, pre)
-                 : tile<8, false, PX, T, false, FOVF>(e, wrs::stage_layout(T, 8, 4, resolve), st, u, p0, d_f, tid, pre);
+        rc = e.code == 2 ? tile<4, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid)
+                         : tile<8, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid);
       } else {
         switch (e.code) {
-        case 0: rc = tile<4, true, PX, T, false, FOVF>(e, wrs::stage_layout(T, 4, 2, resolve), st, u, p0, d_f, tid, pre); break;
-        case 1: rc = tile<8, true, PX, T, false, FOVF>(e, wrs::stage_layout(T, 8, 2, resolve), st, u, p0, d_f, tid, pre); break;
-        case 2: rc = tile<4, false, PX, T, false, FOVF>(e, wrs::stage_layout(T, 4, 4, resolve), st, u, p0, d_f, tid, pre); break;
-        case 3: rc = tile<8, false, PX, T, false, FOVF>(e, wrs::stage_layout(T, 8, 4, resolve), st, u, p0, d_f, tid, pre); break;
-        case 4: rc = tile<0, true, PX, T, false, FOVF>(e, wrs::stage_layout(T, e.s.K, 2, resolve), st, u, p0, d_f, tid); break;
-        case 6: rc = tile<1, true, PX, T, true, FOVF>(e, wrs::stage_layout(T, 1, 2, resolve), st, u, p0, d_f, tid, pre); break;
-        case 7: rc = tile<1, false, PX, T, true, FOVF>(e, wrs::stage_layout(T, 1, 4, resolve), st, u, p0, d_f, tid, pre); break;
-        default: rc = tile<0, false, PX, T, false, FOVF>(e, wrs::stage_layout(T, e.s.K, 4, resolve), st, u, p0, d_f, tid); break;
+          case 0: rc = tile<4, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
+          case 1: rc = tile<8, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
+          case 2: rc = tile<4, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
+          case 3: rc = tile<8, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
+          case 4: rc = tile<0, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
+          case 6: rc = tile<1, true, PX, T, true, FOVF>(e, st, u, px, d_f, tid); break;
+          case 7: rc = tile<1, false, PX, T, true, FOVF>(e, st, u, px, d_f, tid); break;
+          default: rc = tile<0, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
         }
       }
       replaced += rc;

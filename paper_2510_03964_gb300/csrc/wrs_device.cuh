@@ -367,9 +367,8 @@ __device__ __forceinline__ float race_key(float kv, bool flush, bool rescale) {
   return kj;
 }
 
-// Where one group's reservoir planes are read from: global memory (plane
-// stride = plane entries, index = pixel) or a shared-memory tile (stride = tile
-// entries, index = position in the tile). `frame` points at the group's first
+// Where one group's reservoir planes are read from: the global planes (plane
+// stride = plane entries, index = pixel). `frame` points at the group's first
 // RGB triple when the group's colours are contiguous, else is null.
 struct Src {
   const float* W;
@@ -380,7 +379,6 @@ struct Src {
   int64_t stride;
   int64_t at;
   const float* frame;
-  const float* u;  // the group's uniforms (u[0..PX-1]) if already drawn, else null
 };
 
 __device__ __forceinline__ Src global_src(const StreamDev& s, const FrameDev& f, int p0, bool vec) {
@@ -389,7 +387,6 @@ __device__ __forceinline__ Src global_src(const StreamDev& s, const FrameDev& f,
   r.stride = s.plane;
   r.at = p0;
   r.frame = nullptr;
-  r.u = nullptr;
   if (vec) {
     int y, x;
     row_col(s, p0, y, x);
@@ -580,9 +577,8 @@ __device__ __forceinline__ void record_code(const StreamDev& s, const FrameDev& 
 
 // Checked build: the indices a group of PX pixels at p0 uses, against their
 // buffers: state-plane entries p0 .. p0+PX-1 (writes, and reads through
-// global planes), source entries at src.at in planes of src.stride entries
-// (the shared-memory stage or the global planes), the pixels' frame rows and
-// columns and the output. True in the default build.
+// global planes), source entries at src.at in planes of src.stride entries,
+// the pixels' frame rows and columns and the output. True in the default build.
 template <int PX, bool VEC>
 __device__ __forceinline__ bool group_in_bounds(const StreamDev& s, const FrameDev& f, int p0,
                                                 const Src& src, const bool (&valid)[PX],
@@ -596,7 +592,7 @@ __device__ __forceinline__ bool group_in_bounds(const StreamDev& s, const FrameD
     ok = WRS_IN(s, ys[i] >= 0 && ys[i] < s.height && xs[i] >= 0 && xs[i] < s.width &&
                        static_cast<int64_t>(ys[i]) * s.width + xs[i] == static_cast<int64_t>(p0) + i,
                 kChkFrame) && ok;
-    if (f.frame != nullptr && (src.frame == nullptr || src.stride == s.plane))
+    if (f.frame != nullptr)
       ok = WRS_IN(s, static_cast<int64_t>(ys[i]) * f.pitch + 3 * xs[i] + 3 <=
                          static_cast<int64_t>(s.height) * f.pitch,
                   kChkFrame) && ok;
@@ -611,17 +607,15 @@ __device__ __forceinline__ bool group_in_bounds(const StreamDev& s, const FrameD
 }
 
 // One thread's group of PX consecutive pixels p0 .. p0+PX-1 (p0 % PX == 0):
-// weight, key, bias, key race over the K slots, fused resolve, stores. Reads
-// the reservoir through `src` (global planes or a shared-memory tile); writes
-// always go to the global planes. KT > 0 fixes K at compile time. VEC: the
+// weight, key, bias, key race over the K slots, fused resolve, stores; reads
+// and writes the global planes. KT > 0 fixes K at compile time. VEC: the
 // group lies in one row and src.frame / f.out take vector accesses; otherwise
 // every pixel is addressed on its own (and may lie past the end of the image).
 // FOV: a flush map is present (f.fov != null); without one the flush logic is
 // compiled out.
-template <int KT, bool F16, int PX, bool VEC, bool FOV, int KM = FoldCap<KT>::value>
+template <int KT, bool F16, int PX, bool VEC, bool FOV>
 __device__ __forceinline__ int push_group(const StreamDev& s, const FrameDev& f, int p0,
-                                          const Src& src, float d_f,
-                                          const FoldIn<KM>* pre = nullptr) {
+                                          const Src& src, float d_f) {
   const int K = KT > 0 ? KT : s.K;
   const int64_t pl = s.plane;
   const int64_t ss = src.stride;
@@ -676,15 +670,10 @@ __device__ __forceinline__ int push_group(const StreamDev& s, const FrameDev& f,
   // 4 and p0 % PX == 0, so the group never straddles two blocks)
   static_assert(4 % PX == 0, "pixels per thread must divide 4");
   float u[PX];
-  if (src.u != nullptr) {
+  const uint4 blk = philox4x32_10(
+      make_uint4(static_cast<uint32_t>(p0) >> 2, f.t, s.stream_id, 0u), s.seed_lo, s.seed_hi);
 #pragma unroll
-    for (int i = 0; i < PX; ++i) u[i] = src.u[i];
-  } else {
-    const uint4 blk = philox4x32_10(
-        make_uint4(static_cast<uint32_t>(p0) >> 2, f.t, s.stream_id, 0u), s.seed_lo, s.seed_hi);
-#pragma unroll
-    for (int i = 0; i < PX; ++i) u[i] = unit_uniform(word(blk, (p0 + i) & 3));
-  }
+  for (int i = 0; i < PX; ++i) u[i] = unit_uniform(word(blk, (p0 + i) & 3));
 
   // weight (Eq. phat) and A-ES key -ln(u)/w
   float w[PX], k[PX];
@@ -832,7 +821,7 @@ __device__ __forceinline__ int push_group(const StreamDev& s, const FrameDev& f,
       // the sample index goes to the ring as a code
       const uint8_t code = repl[i] ? static_cast<uint8_t>(jm[i] | (flush[i] ? kCodeFlush : 0u))
                                    : (flush[i] ? kCodeFlush : kCodeKeep);
-      record_code<KT, KM>(s, f, p, code, PX == 1 ? pre : nullptr);
+      record_code<KT, FoldCap<KT>::value>(s, f, p, code, nullptr);
     }
   }
   int replaced = 0;
@@ -894,15 +883,10 @@ __device__ __forceinline__ int push_group_literal(const StreamDev& s, const Fram
   for (int i = 0; i < PX; ++i) flush[i] = FOV && valid[i] && f.fov[p0 + i] == 0xFFu;
   static_assert(4 % PX == 0, "pixels per thread must divide 4");
   float u[PX];
-  if (src.u != nullptr) {
+  const uint4 blk = philox4x32_10(
+      make_uint4(static_cast<uint32_t>(p0) >> 2, f.t, s.stream_id, 0u), s.seed_lo, s.seed_hi);
 #pragma unroll
-    for (int i = 0; i < PX; ++i) u[i] = src.u[i];
-  } else {
-    const uint4 blk = philox4x32_10(
-        make_uint4(static_cast<uint32_t>(p0) >> 2, f.t, s.stream_id, 0u), s.seed_lo, s.seed_hi);
-#pragma unroll
-    for (int i = 0; i < PX; ++i) u[i] = unit_uniform(word(blk, (p0 + i) & 3));
-  }
+  for (int i = 0; i < PX; ++i) u[i] = unit_uniform(word(blk, (p0 + i) & 3));
   float w[PX];
 #pragma unroll
   for (int i = 0; i < PX; ++i) w[i] = valid[i] ? pixel_weight(s, d_f, xs[i], ys[i], f.gx, f.gy) : 1.0f;

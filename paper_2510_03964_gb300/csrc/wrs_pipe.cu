@@ -96,23 +96,29 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
                                                       a.extra_tx, ln, FOVF < 0, r.stage_bytes);
                           });
   } else {
+    constexpr int KM = wrs::FoldCap<KT>::value;
     const float d_f = wrs::fovea_density(s);
-    wrs::FoldFor<KT> fin;
-    bool folding = false;
+    // the thread's first pixel moves by a fixed number of rows and columns per
+    // tile: one division for the kernel instead of one per tile
+    const uint32_t jump = static_cast<uint32_t>(step) * T;
+    const int jy = static_cast<int>(jump / static_cast<uint32_t>(s.width));
+    const int jx = static_cast<int>(jump - static_cast<uint32_t>(jy) * s.width);
+    wrs::TilePx<KM> px;
+    px.p = static_cast<uint32_t>(first) * T + tid * PX;
+    px.y = static_cast<int>(px.p / static_cast<uint32_t>(s.width));
+    px.x = static_cast<int>(px.p - static_cast<uint32_t>(px.y) * s.width);
     wrs::consume(
         r, my_tiles, a.timeout_ns, lane,
-        [&](int it) {
-          const int64_t p0 = static_cast<int64_t>(first + it * step) * T;
-          if constexpr (KT > 2) folding = wrs::prefetch_fold<wrs::FoldCap<KT>::value, PX>(s, f, p0, tid, fin);
-        },
-        [&](int it, uint8_t* st, const float* u) {
-          const int64_t p0 = static_cast<int64_t>(first + it * step) * T;
-          const wrs::FoldFor<KT>* pre = folding ? &fin : nullptr;
-          if constexpr (FOVF >= 0)
-            replaced += wrs::compute_tile_fov<KT, F16, PX, T, LIT, FOVF>(s, f, fv, L, st, u, p0,
-                                                                         d_f, tid, pre);
-          else
-            replaced += wrs::compute_tile<KT, F16, PX, T, LIT>(s, f, L, st, u, p0, d_f, tid, pre);
+        [&](int) { wrs::tile_ahead<KM, PX, (KT > 2)>(s, f, px); },
+        [&](int, uint8_t* st, const float* u) {
+          replaced += wrs::compute_tile<KT, F16, PX, T, LIT, FOVF>(s, f, fv, st, u, px, d_f, tid);
+          px.p += jump;
+          px.y += jy;
+          px.x += jx;
+          if (px.x >= s.width) {
+            px.x -= s.width;
+            px.y += 1;
+          }
         });
   }
   __syncthreads();

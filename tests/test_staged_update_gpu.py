@@ -1,0 +1,50 @@
+"""The staged update of the pipelined kernel against the plain kernel, bit for
+bit, where its rare branches meet: states whose bias product is about to be
+rescaled, with empty, equal, zero and largest keys, under flushed pixels, every
+rule, bias and colour precision, with and without the fused resolve."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2510_03964_gb300 as wrs
+
+pytestmark = pytest.mark.gpu
+
+
+def _seeded_state(st, K, hw, rng):
+    raw = st.export_raw()
+    pl, lay = st.layout.plane_px, st.layout
+
+    def plane(off, n):
+        return raw[off: off + 4 * n * pl].view(np.float32).reshape(n, pl)[:, :hw]
+
+    plane(lay.W_off, 1)[:] = rng.choice(np.float32([0.0, 0.5, 3.0, 40.0]), (1, hw))
+    plane(lay.P_off, 1)[:] = rng.choice(np.float32([2.0 ** -64, 1.5 * 2.0 ** -64, 1e-3, 1.0]), (1, hw))
+    plane(lay.key_off, K)[:] = rng.choice(
+        np.float32([np.inf, 0.0, 1e-22, 1e-22, 3e-2, 3e-2, 5e30, 3.4028235e38]), (K, hw))
+    return raw
+
+
+@pytest.mark.parametrize("out", [True, False])
+@pytest.mark.parametrize("bias", [0, 1, 2])
+@pytest.mark.parametrize("K,rule,fp16", [(1, 0, False), (1, 1, False), (1, 1, True), (2, 0, True), (3, 0, False),
+                                         (4, 0, True), (8, 0, False), (8, 0, True), (16, 0, True)])
+def test_rare_branches_equal_the_plain_kernel(K, rule, fp16, bias, out):
+    w, h = 132, 31
+    rng = np.random.default_rng(K + 10 * bias)
+    a, b = (wrs.Stream(w, h, K, 20.0, seed=5, color_fp16=fp16, temporal_bias=bias, update_rule=rule)
+            for _ in range(2))
+    b.set_pipeline(False)
+    raw = _seeded_state(a, K, w * h, rng)
+    outs = [torch.zeros((h, w, 3), device="cuda") for _ in range(2)]
+    for st in (a, b):
+        st.import_raw(raw, 7)
+    for t in range(20):
+        frame = torch.from_numpy(rng.random((h, w, 3), dtype=np.float32)).cuda()
+        fm = torch.from_numpy(rng.choice(np.uint8([0, 3, 255]), (h, w), p=[0.6, 0.35, 0.05])).cuda() if t % 3 else None
+        for st, o in zip((a, b), outs):
+            st.push_frame(frame, (40.0 + t, 11.0), fov_map=fm, out=o if out else None)
+    assert a.check_status() == 0 and b.check_status() == 0
+    assert np.array_equal(a.export_raw()[256:], b.export_raw()[256:])
+    assert a.replacements() == b.replacements()
+    assert torch.equal(outs[0].view(torch.int32), outs[1].view(torch.int32))
