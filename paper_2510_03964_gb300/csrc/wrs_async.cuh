@@ -149,10 +149,11 @@ __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const Fram
 }
 
 // The tile's uniforms, drawn by one warp: one Philox block per 4 pixels,
-// written to u[0 .. T-1].
+// written to u[0 .. T-1], then the warp's arrival on `bar`.
 template <int T>
-__device__ __forceinline__ void draw_tile_uniforms_warp(const StreamDev& s, const FrameDev& f,
-                                                        int64_t p0, float* u, int lane) {
+__device__ __forceinline__ void draw_tile_uniforms(const StreamDev& s, const FrameDev& f,
+                                                   int64_t p0, float* u, uint64_t* bar, int lane) {
+#pragma unroll
   for (int q = lane; q < T / 4; q += 32) {
     const uint32_t blk = static_cast<uint32_t>((p0 >> 2) + q);
     const uint4 b = philox4x32_10(make_uint4(blk, f.t, s.stream_id, 0u), s.seed_lo, s.seed_hi);
@@ -163,6 +164,8 @@ __device__ __forceinline__ void draw_tile_uniforms_warp(const StreamDev& s, cons
     v.w = unit_uniform(b.w);
     reinterpret_cast<float4*>(u)[q] = v;
   }
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar);
 }
 
 // What a consumer thread of a tile knows before the tile has landed: its first
@@ -253,12 +256,12 @@ __device__ __forceinline__ Ring make_ring(uint8_t* smem, uint32_t stage_bytes, i
   return r;
 }
 
-// Thread 0 initialises the barriers (full: one arrival, the producer's;
-// empty: one arrival per consumer warp) and the flag; the caller then
-// synchronises the block.
+// Thread 0 initialises the barriers (full: two arrivals, the copying warp's
+// and the drawing warp's; empty: one arrival per consumer warp) and the flag;
+// the caller then synchronises the block.
 __device__ __forceinline__ void init_ring(const Ring& r, int consumer_warps) {
   for (int i = 0; i < r.S; ++i) {
-    mbar_init(&r.full[i], 1);
+    mbar_init(&r.full[i], 2);
     mbar_init(&r.empty[i], consumer_warps);
   }
   *r.flag = 0;
@@ -273,10 +276,10 @@ __device__ __forceinline__ bool flag_raised(const Ring& r) {
   return *reinterpret_cast<volatile int*>(r.flag) != 0;
 }
 
-// Producer warp: for each of its tiles, waits until the stage is free, draws
-// the tile's uniforms into the stage, arms the stage's full barrier and
-// issues the tile's copies. `tile_fn(it, stage, u, full_bar, lane)` does the
-// drawing and the copies for iteration it. Returns the number of tiles issued.
+// A producer warp: for each of the CTA's tiles, waits until the stage is free
+// and runs `tile_fn(it, stage, u, full_bar, lane)`, which issues the tile's
+// copies (the copying warp) or draws its uniforms (the drawing warp) and
+// arrives on the stage's full barrier. Returns the number of tiles produced.
 template <typename TileFn>
 __device__ __forceinline__ int produce(const Ring& r, int my_tiles, uint64_t timeout_ns, int lane,
                                        TileFn tile_fn) {

@@ -60,7 +60,7 @@ __device__ __forceinline__ bool entry_f16(const BatchEntry& e) {
 }
 
 constexpr int kConsumerWarps = 8;
-constexpr int kBatchThreads = (kConsumerWarps + 1) * 32;
+constexpr int kBatchThreads = (kConsumerWarps + 2) * 32;
 
 // Adds a warp's running count of replacements in entry ei to the CTA's
 // per-stream total and clears it: once per stream a warp leaves, not per tile.
@@ -86,23 +86,20 @@ __device__ __forceinline__ int tile(const BatchEntry& e, uint8_t* st, const floa
   return wrs::compute_tile<KT, F16, PX, T, LIT, FOVF>(e.s, e.f, e.fv, st, u, px, d_f, tid);
 }
 
-// The producer's work for one tile of entry e: its uniforms, then its bulk
-// copies. KT, CS > 0 fix the slot count and colour bytes at compile time (the
+// The copying warp's work for one tile of entry e. KT, CS > 0 fix the slot count and colour bytes at compile time (the
 // K = 4 / 8 families), so the copy sizes and stage offsets fold to constants.
 template <int T, int KT, int CS, bool COPY_FRAME>
-__device__ __forceinline__ void produce_tile(const BatchEntry& e, int64_t p0, uint8_t* st, float* u,
+__device__ __forceinline__ void produce_tile(const BatchEntry& e, int64_t p0, uint8_t* st,
                                              uint64_t* full, int ln, uint32_t stage_cap) {
   const int K = KT > 0 ? KT : e.s.K;
   const int cs = CS > 0 ? CS : (entry_f16(e) ? 2 : 4);
   const bool resolve = stage_records(e);
   const StageLayout L = wrs::stage_layout(T, K, cs, resolve);
-  wrs::draw_tile_uniforms_warp<T>(e.s, e.f, p0, u, ln);
-  __syncwarp();
   wrs::issue_tile_copies<T>(e.s, e.f, K, cs, resolve, L, st, full, p0, 0u, ln, COPY_FRAME, stage_cap);
 }
 
-// Warp-specialised like the single-stream pipelined kernel: warp 8 draws each
-// tile's uniforms and issues its copies, warps 0..7 compute it. FOVF >= 0:
+// Warp-specialised like the single-stream pipelined kernel: warp 8 issues each
+// tile's copies, warp 9 draws its uniforms, warps 0..7 compute it. FOVF >= 0:
 // no frame is copied; the consumers foveate each pixel from the stream's
 // image and mip levels (filter FOVF, WRS_FILTER_*) into the stage first.
 template <int PX, int FAM, int FOVF = -1>
@@ -135,22 +132,31 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
   if (warp == kConsumerWarps) {
     int pe = 0;  // entry of the producer's current tile
     issued = wrs::produce(r, my_tiles, a.timeout_ns, lane,
-                          [&](int it, uint8_t* st, float* u, uint64_t* full, int ln) {
+                          [&](int it, uint8_t* st, float*, uint64_t* full, int ln) {
                             const int g = first + it * step;
                             pe = entry_after(a, g, pe);
                             const BatchEntry& e = a.e[pe];
                             const int64_t p0 = static_cast<int64_t>(g - e.tile0) * T;
                             constexpr bool cf = FOVF < 0;
                             if constexpr (FAM == kFamF16K48) {
-                              if (e.code == 0) produce_tile<T, 4, 2, cf>(e, p0, st, u, full, ln, r.stage_bytes);
-                              else produce_tile<T, 8, 2, cf>(e, p0, st, u, full, ln, r.stage_bytes);
+                              if (e.code == 0) produce_tile<T, 4, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
+                              else produce_tile<T, 8, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
                             } else if constexpr (FAM == kFamF32K48) {
-                              if (e.code == 2) produce_tile<T, 4, 4, cf>(e, p0, st, u, full, ln, r.stage_bytes);
-                              else produce_tile<T, 8, 4, cf>(e, p0, st, u, full, ln, r.stage_bytes);
+                              if (e.code == 2) produce_tile<T, 4, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
+                              else produce_tile<T, 8, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
                             } else {
-                              produce_tile<T, 0, 0, cf>(e, p0, st, u, full, ln, r.stage_bytes);
+                              produce_tile<T, 0, 0, cf>(e, p0, st, full, ln, r.stage_bytes);
                             }
                           });
+  } else if (warp == kConsumerWarps + 1) {
+    int pe = 0;
+    wrs::produce(r, my_tiles, a.timeout_ns, lane,
+                 [&](int it, uint8_t*, float* u, uint64_t* full, int ln) {
+                   const int g = first + it * step;
+                   pe = entry_after(a, g, pe);
+                   const BatchEntry& e = a.e[pe];
+                   wrs::draw_tile_uniforms<T>(e.s, e.f, static_cast<int64_t>(g - e.tile0) * T, u, full, ln);
+                 });
   } else {
     wrs::TilePx<8> px;
     int ei = 0;        // entry of the consumer's current tile

@@ -1,12 +1,15 @@
 // Pipelined persistent form of the fused update + resolve (sm_103a).
 //
 // Persistent CTAs (one or more per SM) walk the image in tiles of
-// T = 256 * PX pixels. A producer warp streams the planes a tile needs (frame
-// RGB, W, P, the K key planes and, for the fused resolve, the K weight and 3K
-// colour planes) into a ring of S shared-memory stages with 1-D bulk
-// asynchronous copies (cp.async.bulk) that complete on one transaction-count
-// "full" mbarrier per stage, after drawing the tile's uniforms (one Philox
-// block per 4 pixels) into the stage. Eight consumer warps compute each
+// T = 256 * PX pixels. A copying warp streams the planes a tile needs (frame
+// RGB, W, P, the K key planes and, for the fused resolve, the K slot records)
+// into a ring of S shared-memory stages with 1-D bulk asynchronous copies
+// (cp.async.bulk) that complete on one transaction-count "full" mbarrier per
+// stage; a drawing warp adds the tile's uniforms (one Philox block per 4
+// pixels). With one warp doing both, the draw (about 220 dependent
+// instructions a tile) held back the copies: 4K K = 8 FP16 244 -> 238 us, 4K
+// literal rule 73.8 -> 69.7 us, 8-stream FP16 batch 990 -> 932 us when the
+// drawing moved to its own warp. Eight consumer warps compute each
 // landed tile from shared memory with the same per-pixel code as the plain
 // kernel (bit-identical results), write straight to global memory and free
 // the stage through its "empty" mbarrier. No block-wide barrier sits inside
@@ -42,11 +45,11 @@ struct PipeArgs {
 };
 
 constexpr int kConsumerWarps = 8;
-constexpr int kPipeThreads = (kConsumerWarps + 1) * 32;
+constexpr int kPipeThreads = (kConsumerWarps + 2) * 32;
 
 // Warp-specialised: warps 0..7 compute (consumers, PX pixels per thread), warp 8
-// draws uniforms and issues copies (producer). Consumers and producer meet
-// only at the per-stage full/empty barriers, never at a block-wide barrier.
+// issues copies and warp 9 draws uniforms. They meet only at the per-stage
+// full/empty barriers, never at a block-wide barrier.
 // FOVF >= 0: the frame is not copied but foveated by the consumers from `fv`
 // with filter FOVF (WRS_FILTER_*) as they compute; FOVF < 0: `fv` is unused.
 // Resident CTAs per SM the compiler is asked to fit: three for one or two
@@ -88,13 +91,16 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
   int replaced = 0;
   if (warp == kConsumerWarps) {
     issued = wrs::produce(r, my_tiles, a.timeout_ns, lane,
-                          [&](int it, uint8_t* st, float* u, uint64_t* full, int ln) {
+                          [&](int it, uint8_t* st, float*, uint64_t* full, int ln) {
                             const int64_t p0 = static_cast<int64_t>(first + it * step) * T;
-                            wrs::draw_tile_uniforms_warp<T>(s, f, p0, u, ln);
-                            __syncwarp();
                             wrs::issue_tile_copies<T>(s, f, K, cs, resolve, L, st, full, p0,
                                                       a.extra_tx, ln, FOVF < 0, r.stage_bytes);
                           });
+  } else if (warp == kConsumerWarps + 1) {
+    wrs::produce(r, my_tiles, a.timeout_ns, lane,
+                 [&](int it, uint8_t*, float* u, uint64_t* full, int ln) {
+                   wrs::draw_tile_uniforms<T>(s, f, static_cast<int64_t>(first + it * step) * T, u, full, ln);
+                 });
   } else {
     constexpr int KM = wrs::FoldCap<KT>::value;
     const float d_f = wrs::fovea_density(s);
