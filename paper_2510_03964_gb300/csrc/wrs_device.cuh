@@ -524,29 +524,67 @@ __device__ __forceinline__ void fold_load(const StreamDev& s, const uint32_t* id
                  (static_cast<uint32_t>(b[4 * w + 3]) << 24);
 }
 
+// Left shifts that give 0 for amounts of 32 and above (and for negative ones).
+__device__ __forceinline__ uint32_t shl_or_0(uint32_t v, uint32_t n) {
+  uint32_t r;
+  asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+  return r;
+}
+
 // Applies the loaded codes of frames lo .. t-1 (older ring entries, and
 // entries of frames before lo, are skipped) and then, if c_now is not
 // kCodeKeep, code c_now of frame t; writes pixel p's K indices to `idx`.
+//
+// With up to 8 slots and no flush among the codes, the frame that took slot j
+// last is kept as byte j of a 64-bit word: a code c puts its frame's number
+// (0..15, from t-15) at bit 8c, and kCodeKeep shifts out of both halves. That
+// costs a fold about 10 instructions per code instead of 4 per code and slot:
+// VR K = 8 FP16 with the full bias 151 -> 138 us, HD K = 4 48.3 -> 46.9 us.
 template <int KM>
 __device__ __forceinline__ void fold_store(const StreamDev& s, uint32_t* idx, int K, uint32_t t,
                                            uint32_t lo, int64_t p, const FoldIn<KM>& in,
                                            uint8_t c_now) {
   const int64_t pl = s.plane;
+  uint32_t code[kRingFrames / 4];
+#pragma unroll
+  for (int w = 0; w < kRingFrames / 4; ++w) code[w] = in.code[w];
+  code[kRingFrames / 4 - 1] = (code[kRingFrames / 4 - 1] & 0x00ffffffu) | (static_cast<uint32_t>(c_now) << 24);
+  // frames before lo keep (t - lo <= 15 frames are pending)
+  const uint32_t skip = kRingFrames - 1 - (t - lo);
+#pragma unroll
+  for (int w = 0; w < kRingFrames / 4; ++w) {
+    if (skip >= 4u * w + 4u) code[w] = 0xffffffffu;
+    else if (skip > 4u * w) code[w] |= 0xffffffffu >> (32u - 8u * (skip - 4u * w));
+  }
+  // a flush code has bit 7 set and bit 6 clear, kCodeKeep has both set
+  uint32_t flushed = 0;
+#pragma unroll
+  for (int w = 0; w < kRingFrames / 4; ++w) flushed |= code[w] & ~(code[w] << 1) & 0x80808080u;
   uint32_t v[KM];
 #pragma unroll
   for (int j = 0; j < KM; ++j) v[j] = in.v[j];
+  const uint32_t first = t - static_cast<uint32_t>(kRingFrames - 1);
+  if (KM <= 8 && flushed == 0u) {
+    uint32_t last0 = 0xffffffffu, last1 = 0xffffffffu;
 #pragma unroll
-  for (int k = 0; k < kRingFrames - 1; ++k) {
-    const uint32_t fr = t - static_cast<uint32_t>(kRingFrames - 1) + k;
-    const uint8_t c = static_cast<uint8_t>(in.code[k >> 2] >> (8 * (k & 3)));
-    if (fr >= lo && fr < t && c != kCodeKeep) {
-#pragma unroll
-      for (int j = 0; j < KM; ++j) v[j] = after_code(v[j], j, c, fr);
+    for (int k = 0; k < kRingFrames; ++k) {
+      const uint32_t at = 8u * ((code[k >> 2] >> (8 * (k & 3))) & 0xffu);
+      last0 = (last0 & ~shl_or_0(0xffu, at)) | shl_or_0(k, at);
+      if (KM > 4) last1 = (last1 & ~shl_or_0(0xffu, at - 32u)) | shl_or_0(k, at - 32u);
     }
-  }
-  if (c_now != kCodeKeep) {
 #pragma unroll
-    for (int j = 0; j < KM; ++j) v[j] = after_code(v[j], j, c_now, t);
+    for (int j = 0; j < KM; ++j) {
+      const uint32_t k = ((j < 4 ? last0 : last1) >> (8 * (j & 3))) & 0xffu;
+      if (k != 0xffu) v[j] = first + k;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < kRingFrames; ++k) {
+      const uint8_t c = static_cast<uint8_t>(code[k >> 2] >> (8 * (k & 3)));
+      if (c == kCodeKeep) continue;
+#pragma unroll
+      for (int j = 0; j < KM; ++j) v[j] = after_code(v[j], j, c, first + k);
+    }
   }
 #pragma unroll
   for (int j = 0; j < KM; ++j)
