@@ -205,7 +205,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     e.f.t = x->t;
     e.f.map_lo = wrs_map_lo(x);
     e.status = wrs_status_word(x);
-    e.tile0 = static_cast<int>(tiles);
+    e.tile0 = static_cast<uint32_t>(tiles);
     e.code = code_of(x->cfg);
     tiles += (static_cast<int64_t>(e.s.hw) + T - 1) / T;
     const bool records = out != nullptr || x->cfg.temporal_bias == 2;
@@ -222,11 +222,10 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
       --stages;
     while (stages > 1 && wrs::ring_bytes(stage_bytes, T, stages) > kSmemBudget) --stages;
   }
-  const size_t smem = wrs::ring_bytes(stage_bytes, T, stages);
+  size_t smem = wrs::ring_bytes(stage_bytes, T, stages);
   if (smem > kSmemBudget)
     return wrs_fail(WRS_ERR_ARG, "%d stages of %u B exceed shared memory", stages, stage_bytes);
   a.n = n;
-  a.ntiles = static_cast<int>(tiles);
   a.stages = stages;
   a.stage_bytes = stage_bytes;
   a.timeout_ns = ctxs[0]->timeout_ns;
@@ -258,15 +257,14 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, fn, kBatchThreads, smem);
   if (e != cudaSuccess) return wrs_cuda_fail(e, "push_batch: occupancy");
   if (fit < 1) return wrs_fail(WRS_ERR_ARG, "batch kernel does not fit on an SM");
-  const int per_sm = b->ctas_per_sm > 0 && b->ctas_per_sm < fit ? b->ctas_per_sm : fit;
-  const int64_t want = static_cast<int64_t>(ctxs[0]->sms) * per_sm;
-  const int grid = static_cast<int>(tiles < want ? tiles : want);
+  // fewer CTAs per SM than fit: a larger shared-memory request keeps the others out
+  if (b->ctas_per_sm > 0 && b->ctas_per_sm < fit) smem = wrs::smem_for_ctas(smem, b->ctas_per_sm);
 
   cudaKernelNodeParams kp;
   std::memset(&kp, 0, sizeof kp);
   void* params[1] = {&a};
   kp.func = const_cast<void*>(fn);
-  kp.gridDim = dim3(grid);
+  kp.gridDim = dim3(static_cast<unsigned>(tiles));  // one CTA per tile: see request_tile
   kp.blockDim = dim3(kBatchThreads);
   kp.sharedMemBytes = static_cast<unsigned>(smem);
   kp.kernelParams = params;

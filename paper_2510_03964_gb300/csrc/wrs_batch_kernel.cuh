@@ -24,7 +24,7 @@ struct BatchEntry {
   FrameDev f;
   wrs::FovDev fv;  // the stream's rendered image and mip levels (foveating batches only)
   uint32_t* status;
-  int tile0;   // first global tile of this stream
+  uint32_t tile0;  // first global tile of this stream
   int code;    // arithmetic variant: 0 K=4 f16, 1 K=8 f16, 2 K=4 f32, 3 K=8 f32, 4 any K f16,
                // 5 any K f32, 6 literal f16, 7 literal f32
 };
@@ -37,7 +37,6 @@ __device__ __forceinline__ bool stage_records(const BatchEntry& e) {
 
 struct BatchArgs {
   int n;
-  int ntiles;
   int stages;
   uint32_t stage_bytes;  // largest stage of any stream in the batch
   uint64_t timeout_ns;
@@ -50,7 +49,7 @@ static_assert(sizeof(BatchArgs) <= 32000, "batch descriptor too large for a kern
 // visits its tiles in ascending order, so each of its warps keeps the entry of
 // its previous tile in `e` and moves it forward (a few steps per stream
 // boundary instead of a search per tile).
-__device__ __forceinline__ int entry_after(const BatchArgs& a, int g, int e) {
+__device__ __forceinline__ int entry_after(const BatchArgs& a, uint32_t g, int e) {
   while (e + 1 < a.n && a.e[e + 1].tile0 <= g) ++e;
   return e;
 }
@@ -126,50 +125,45 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
   }
   __syncthreads();
 
-  const int first = blockIdx.x, step = gridDim.x;
-  const int my_tiles = first < a.ntiles ? (a.ntiles - 1 - first) / step + 1 : 0;
   int issued = 0;
   if (warp == kConsumerWarps) {
-    int pe = 0;  // entry of the producer's current tile
-    issued = wrs::produce(r, my_tiles, a.timeout_ns, lane,
-                          [&](int it, uint8_t* st, float*, uint64_t* full, int ln) {
-                            const int g = first + it * step;
-                            pe = entry_after(a, g, pe);
-                            const BatchEntry& e = a.e[pe];
-                            const int64_t p0 = static_cast<int64_t>(g - e.tile0) * T;
-                            constexpr bool cf = FOVF < 0;
-                            if constexpr (FAM == kFamF16K48) {
-                              if (e.code == 0) produce_tile<T, 4, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
-                              else produce_tile<T, 8, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
-                            } else if constexpr (FAM == kFamF32K48) {
-                              if (e.code == 2) produce_tile<T, 4, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
-                              else produce_tile<T, 8, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
-                            } else {
-                              produce_tile<T, 0, 0, cf>(e, p0, st, full, ln, r.stage_bytes);
-                            }
-                          });
+    int pe = 0;  // entry of the copying warp's current tile
+    issued = wrs::produce<true>(r, a.timeout_ns, lane,
+                                [&](uint32_t g, uint8_t* st, float*, uint64_t* full, int ln) {
+      pe = entry_after(a, g, pe);
+      const BatchEntry& e = a.e[pe];
+      const int64_t p0 = static_cast<int64_t>(g - e.tile0) * T;
+      constexpr bool cf = FOVF < 0;
+      if constexpr (FAM == kFamF16K48) {
+        if (e.code == 0) produce_tile<T, 4, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
+        else produce_tile<T, 8, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
+      } else if constexpr (FAM == kFamF32K48) {
+        if (e.code == 2) produce_tile<T, 4, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
+        else produce_tile<T, 8, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
+      } else {
+        produce_tile<T, 0, 0, cf>(e, p0, st, full, ln, r.stage_bytes);
+      }
+    });
   } else if (warp == kConsumerWarps + 1) {
     int pe = 0;
-    wrs::produce(r, my_tiles, a.timeout_ns, lane,
-                 [&](int it, uint8_t*, float* u, uint64_t* full, int ln) {
-                   const int g = first + it * step;
-                   pe = entry_after(a, g, pe);
-                   const BatchEntry& e = a.e[pe];
-                   wrs::draw_tile_uniforms<T>(e.s, e.f, static_cast<int64_t>(g - e.tile0) * T, u, full, ln);
-                 });
+    wrs::produce<false>(r, a.timeout_ns, lane,
+                        [&](uint32_t g, uint8_t*, float* u, uint64_t* full, int ln) {
+      pe = entry_after(a, g, pe);
+      const BatchEntry& e = a.e[pe];
+      wrs::draw_tile_uniforms<T>(e.s, e.f, static_cast<int64_t>(g - e.tile0) * T, u, full, ln);
+    });
   } else {
     wrs::TilePx<8> px;
     int ei = 0;        // entry of the consumer's current tile
     int replaced = 0;  // this thread's replacements in entry ei so far
-    wrs::consume(r, my_tiles, a.timeout_ns, lane, [&](int it) {
-      const int g = first + it * step;
+    wrs::consume(r, a.timeout_ns, lane, [&](uint32_t g) {
       const int next = entry_after(a, g, ei);
       if (next != ei) {
         flush_count(replaced_s, ei, replaced, lane);
         ei = next;
       }
       const BatchEntry& e = a.e[ei];
-      px.p = static_cast<uint32_t>(g - e.tile0) * T + tid * PX;
+      px.p = (g - e.tile0) * T + tid * PX;
       wrs::row_col(e.s, static_cast<int>(px.p), px.y, px.x);
       // fold inputs only for entries that compute with K = 4 or 8
       if (e.code < 4) {
@@ -177,7 +171,7 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
       } else {
         wrs::tile_ahead<8, PX, false>(e.s, e.f, px);
       }
-    }, [&](int, uint8_t* st, const float* u) {
+    }, [&](uint8_t* st, const float* u) {
       const BatchEntry& e = a.e[ei];
       const float d_f = d_f_s[ei];
       if (failed_s[ei] != 0) return;

@@ -457,8 +457,8 @@ extern "C" int wrs_push_frame(wrs_ctx* x, const float* d_frame, int64_t pitch, f
   f.map_lo = wrs_map_lo(x);
   cudaError_t e;
   if (x->pipe && wrs_pipe_supported(x, d_frame, pitch, d_out)) {
-    e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, x->pipe_px, x->pipe_stages, x->sms,
-                        x->pipe_ctas, wrs_status_word(x), x->timeout_ns, x->test_extra_tx,
+    e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, x->pipe_px, x->pipe_stages, x->pipe_ctas,
+                        wrs_status_word(x), x->timeout_ns, x->test_extra_tx,
                         static_cast<cudaStream_t>(stream));
   } else {
     const int px = wrs_effective_px(x, d_frame, pitch, d_out);
@@ -501,8 +501,8 @@ extern "C" int wrs_push_foveated(wrs_ctx* x, const float* d_img, int64_t img_pit
   int px = x->pipe_px, stages = x->pipe_stages;
   // the foveating form takes one pixel per thread: its own stage count then
   if (px != 1) stages = wrs_default_stages(x->cfg.K, x->cfg.color_fp16 != 0, 1);
-  cudaError_t e = wrs_launch_pipe_fov(s, f, fv, filter, x->cfg.color_fp16 != 0, stages, x->sms,
-                                      x->pipe_ctas, wrs_status_word(x), x->timeout_ns,
+  cudaError_t e = wrs_launch_pipe_fov(s, f, fv, filter, x->cfg.color_fp16 != 0, stages, x->pipe_ctas,
+                                      wrs_status_word(x), x->timeout_ns,
                                       static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return wrs_cuda_fail(e, "wrs_push_foveated: launch");
   x->t += 1;

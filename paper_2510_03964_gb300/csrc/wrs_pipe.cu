@@ -37,7 +37,6 @@ namespace {
 
 struct PipeArgs {
   int stages;
-  int ntiles;
   int resolve;             // copy weight/colour planes (fused resolve or full temporal bias)
   uint32_t* status;        // stream status word (WRS_OK or WRS_ERR_TIMEOUT)
   uint64_t timeout_ns;
@@ -84,47 +83,33 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
   __syncthreads();
   if (failed != 0) return;
 
-  const int first = blockIdx.x;
-  const int step = gridDim.x;
-  const int my_tiles = first < a.ntiles ? (a.ntiles - 1 - first) / step + 1 : 0;
   int issued = 0;
   int replaced = 0;
   if (warp == kConsumerWarps) {
-    issued = wrs::produce(r, my_tiles, a.timeout_ns, lane,
-                          [&](int it, uint8_t* st, float*, uint64_t* full, int ln) {
-                            const int64_t p0 = static_cast<int64_t>(first + it * step) * T;
-                            wrs::issue_tile_copies<T>(s, f, K, cs, resolve, L, st, full, p0,
-                                                      a.extra_tx, ln, FOVF < 0, r.stage_bytes);
-                          });
+    issued = wrs::produce<true>(r, a.timeout_ns, lane,
+                                [&](uint32_t tile, uint8_t* st, float*, uint64_t* full, int ln) {
+                                  wrs::issue_tile_copies<T>(s, f, K, cs, resolve, L, st, full,
+                                                            static_cast<int64_t>(tile) * T, a.extra_tx,
+                                                            ln, FOVF < 0, r.stage_bytes);
+                                });
   } else if (warp == kConsumerWarps + 1) {
-    wrs::produce(r, my_tiles, a.timeout_ns, lane,
-                 [&](int it, uint8_t*, float* u, uint64_t* full, int ln) {
-                   wrs::draw_tile_uniforms<T>(s, f, static_cast<int64_t>(first + it * step) * T, u, full, ln);
-                 });
+    wrs::produce<false>(r, a.timeout_ns, lane,
+                        [&](uint32_t tile, uint8_t*, float* u, uint64_t* full, int ln) {
+                          wrs::draw_tile_uniforms<T>(s, f, static_cast<int64_t>(tile) * T, u, full, ln);
+                        });
   } else {
     constexpr int KM = wrs::FoldCap<KT>::value;
     const float d_f = wrs::fovea_density(s);
-    // the thread's first pixel moves by a fixed number of rows and columns per
-    // tile: one division for the kernel instead of one per tile
-    const uint32_t jump = static_cast<uint32_t>(step) * T;
-    const int jy = static_cast<int>(jump / static_cast<uint32_t>(s.width));
-    const int jx = static_cast<int>(jump - static_cast<uint32_t>(jy) * s.width);
     wrs::TilePx<KM> px;
-    px.p = static_cast<uint32_t>(first) * T + tid * PX;
-    px.y = static_cast<int>(px.p / static_cast<uint32_t>(s.width));
-    px.x = static_cast<int>(px.p - static_cast<uint32_t>(px.y) * s.width);
     wrs::consume(
-        r, my_tiles, a.timeout_ns, lane,
-        [&](int) { wrs::tile_ahead<KM, PX, (KT > 2)>(s, f, px); },
-        [&](int, uint8_t* st, const float* u) {
+        r, a.timeout_ns, lane,
+        [&](uint32_t tile) {
+          px.p = tile * T + tid * PX;
+          wrs::row_col(s, static_cast<int>(px.p), px.y, px.x);
+          wrs::tile_ahead<KM, PX, (KT > 2)>(s, f, px);
+        },
+        [&](uint8_t* st, const float* u) {
           replaced += wrs::compute_tile<KT, F16, PX, T, LIT, FOVF>(s, f, fv, st, u, px, d_f, tid);
-          px.p += jump;
-          px.y += jy;
-          px.x += jx;
-          if (px.x >= s.width) {
-            px.x -= s.width;
-            px.y += 1;
-          }
         });
   }
   __syncthreads();
@@ -136,14 +121,13 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
 }
 
 template <int KT, bool F16, int PX, bool LIT = false, int FOVF = -1>
-cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int sms,
-                          int ctas_per_sm, cudaStream_t st, const FovDev& fv = FovDev{}) {
+cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int ctas_per_sm,
+                          cudaStream_t st, const FovDev& fv = FovDev{}) {
   constexpr int T = kConsumerWarps * 32 * PX;
   const StageLayout L = wrs::stage_layout(T, s.K, F16 ? 2 : 4, a.resolve != 0);
-  const size_t smem = wrs::ring_bytes(L.bytes, T, a.stages);
-  // per instantiation and device: the largest dynamic shared memory already
-  // allowed; the lock keeps two host threads from lowering each other's limit
-  static size_t configured[64] = {};
+  size_t smem = wrs::ring_bytes(L.bytes, T, a.stages);
+  // per instantiation and device: the whole budget allowed once
+  static bool configured[64] = {};
   static std::mutex lock;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -151,11 +135,11 @@ cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   {
     std::lock_guard<std::mutex> hold(lock);
-    if (smem > configured[dev]) {
+    if (!configured[dev]) {
       e = cudaFuncSetAttribute(pipe_kernel<KT, F16, PX, LIT, FOVF>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBudget));
       if (e != cudaSuccess) return e;
-      configured[dev] = smem;
+      configured[dev] = true;
     }
   }
   int fit = 0;
@@ -163,11 +147,10 @@ cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int
                                                     kPipeThreads, smem);
   if (e != cudaSuccess) return e;
   if (fit < 1) return cudaErrorInvalidConfiguration;
-  const int per_sm = ctas_per_sm > 0 && ctas_per_sm < fit ? ctas_per_sm : fit;
-  a.ntiles = static_cast<int>((static_cast<int64_t>(s.hw) + T - 1) / T);
-  const int64_t want = static_cast<int64_t>(sms) * per_sm;
-  const int grid = static_cast<int>(a.ntiles < want ? a.ntiles : want);
-  pipe_kernel<KT, F16, PX, LIT, FOVF><<<grid, kPipeThreads, smem, st>>>(s, f, a, fv);
+  // fewer CTAs per SM than fit: a larger shared-memory request keeps the others out
+  if (ctas_per_sm > 0 && ctas_per_sm < fit) smem = wrs::smem_for_ctas(smem, ctas_per_sm);
+  const int64_t tiles = (static_cast<int64_t>(s.hw) + T - 1) / T;
+  pipe_kernel<KT, F16, PX, LIT, FOVF><<<static_cast<unsigned>(tiles), kPipeThreads, smem, st>>>(s, f, a, fv);
   return cudaGetLastError();
 }
 
@@ -175,35 +158,35 @@ cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int
 // any other through the generic instantiation, and the literal rule.
 template <bool F16, int FILTER>
 cudaError_t launch_pipe_fov_k(const StreamDev& s, const FrameDev& f, const FovDev& fv,
-                              const PipeArgs& a, int sms, int ctas, cudaStream_t st) {
-  if (s.literal) return launch_pipe_t<1, F16, 1, true, FILTER>(s, f, a, sms, ctas, st, fv);
+                              const PipeArgs& a, int ctas, cudaStream_t st) {
+  if (s.literal) return launch_pipe_t<1, F16, 1, true, FILTER>(s, f, a, ctas, st, fv);
   switch (s.K) {
-    case 4: return launch_pipe_t<4, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
-    case 8: return launch_pipe_t<8, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
-    default: return launch_pipe_t<0, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
+    case 4: return launch_pipe_t<4, F16, 1, false, FILTER>(s, f, a, ctas, st, fv);
+    case 8: return launch_pipe_t<8, F16, 1, false, FILTER>(s, f, a, ctas, st, fv);
+    default: return launch_pipe_t<0, F16, 1, false, FILTER>(s, f, a, ctas, st, fv);
   }
 }
 
 template <int KT, bool F16, bool LIT = false>
-cudaError_t launch_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px,
-                           int sms, int ctas, cudaStream_t st) {
+cudaError_t launch_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int ctas,
+                            cudaStream_t st) {
   switch (px) {
-    case 4: return launch_pipe_t<KT, F16, 4, LIT>(s, f, a, sms, ctas, st);
-    case 2: return launch_pipe_t<KT, F16, 2, LIT>(s, f, a, sms, ctas, st);
-    default: return launch_pipe_t<KT, F16, 1, LIT>(s, f, a, sms, ctas, st);
+    case 4: return launch_pipe_t<KT, F16, 4, LIT>(s, f, a, ctas, st);
+    case 2: return launch_pipe_t<KT, F16, 2, LIT>(s, f, a, ctas, st);
+    default: return launch_pipe_t<KT, F16, 1, LIT>(s, f, a, ctas, st);
   }
 }
 
 template <bool F16>
-cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px,
-                          int sms, int ctas, cudaStream_t st) {
-  if (s.literal) return launch_pipe_px<1, F16, true>(s, f, a, px, sms, ctas, st);
+cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int ctas,
+                           cudaStream_t st) {
+  if (s.literal) return launch_pipe_px<1, F16, true>(s, f, a, px, ctas, st);
   switch (s.K) {
-    case 1: return launch_pipe_px<1, F16>(s, f, a, px, sms, ctas, st);
-    case 2: return launch_pipe_px<2, F16>(s, f, a, px, sms, ctas, st);
-    case 4: return launch_pipe_px<4, F16>(s, f, a, px, sms, ctas, st);
-    case 8: return launch_pipe_px<8, F16>(s, f, a, px, sms, ctas, st);
-    default: return launch_pipe_px<0, F16>(s, f, a, px, sms, ctas, st);
+    case 1: return launch_pipe_px<1, F16>(s, f, a, px, ctas, st);
+    case 2: return launch_pipe_px<2, F16>(s, f, a, px, ctas, st);
+    case 4: return launch_pipe_px<4, F16>(s, f, a, px, ctas, st);
+    case 8: return launch_pipe_px<8, F16>(s, f, a, px, ctas, st);
+    default: return launch_pipe_px<0, F16>(s, f, a, px, ctas, st);
   }
 }
 
@@ -222,32 +205,30 @@ bool wrs_pipe_supported(const wrs_ctx* x, const float* frame, int64_t pitch, con
 }
 
 cudaError_t wrs_launch_pipe_fov(const StreamDev& s, const FrameDev& f, const FovDev& fv, int filter,
-                                bool f16, int stages, int sms, int ctas_per_sm, uint32_t* status,
+                                bool f16, int stages, int ctas_per_sm, uint32_t* status,
                                 uint64_t timeout_ns, cudaStream_t st) {
   PipeArgs a;
   a.stages = stages;
-  a.ntiles = 0;
   a.resolve = (f.out != nullptr || s.bias == 2) ? 1 : 0;  // records: resolve or Delta L
   a.status = status;
   a.timeout_ns = timeout_ns;
   a.extra_tx = 0;
   if (filter == WRS_FILTER_BOX)
-    return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, st)
-               : launch_pipe_fov_k<false, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, st);
-  return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, st)
-             : launch_pipe_fov_k<false, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, st);
+    return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BOX>(s, f, fv, a, ctas_per_sm, st)
+               : launch_pipe_fov_k<false, WRS_FILTER_BOX>(s, f, fv, a, ctas_per_sm, st);
+  return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BILINEAR>(s, f, fv, a, ctas_per_sm, st)
+             : launch_pipe_fov_k<false, WRS_FILTER_BILINEAR>(s, f, fv, a, ctas_per_sm, st);
 }
 
 cudaError_t wrs_launch_pipe(const StreamDev& s, const FrameDev& f, bool f16, int px, int stages,
-                            int sms, int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
+                            int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
                             uint32_t extra_tx, cudaStream_t st) {
   PipeArgs a;
   a.stages = stages;
-  a.ntiles = 0;
   a.resolve = (f.out != nullptr || s.bias == 2) ? 1 : 0;  // records: resolve or Delta L
   a.status = status;
   a.timeout_ns = timeout_ns;
   a.extra_tx = extra_tx;
-  return f16 ? launch_pipe_k<true>(s, f, a, px, sms, ctas_per_sm, st)
-             : launch_pipe_k<false>(s, f, a, px, sms, ctas_per_sm, st);
+  return f16 ? launch_pipe_k<true>(s, f, a, px, ctas_per_sm, st)
+             : launch_pipe_k<false>(s, f, a, px, ctas_per_sm, st);
 }
