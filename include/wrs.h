@@ -275,8 +275,9 @@ int wrs_set_launch(wrs_ctx* ctx, int block_threads, int px_per_thread);
 int wrs_get_launch(const wrs_ctx* ctx, int* block_threads, int* px_per_thread);
 
 /* Kernel choice for wrs_push_frame. enable = 1 (default) uses the pipelined
- * persistent kernel whenever width % 4 == 0, frame_pitch_elems == 3 * width and
- * frame/out are 16-byte aligned (else the plain kernel runs): persistent CTAs
+ * persistent kernel whenever frame_pitch_elems == 3 * width and frame/out are
+ * 16-byte aligned (else the plain kernel runs; where width % 4 != 0 it takes
+ * one pixel per thread whatever was asked for): persistent CTAs
  * (ctas_per_sm per SM; 0 = as many as registers and shared memory allow)
  * stream tiles of 256 * px_per_thread pixels (1, 2 or 4) through `stages`
  * shared-memory stages with bulk asynchronous copies. 0 for px_per_thread

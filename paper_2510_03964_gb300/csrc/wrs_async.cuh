@@ -79,8 +79,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // Warp-wide: lane 0 arms `bar` for the tile's bytes (plus extra_tx, which is
 // non-zero only to test the timeout path), then the lanes issue one bulk copy
 // per plane segment. The tile starts at pixel p0 (a multiple of T >= 256);
-// requires frame rows without padding, width % 4 == 0 and 16-byte aligned
-// frame and state planes. copy_frame = false leaves the frame segment to the
+// requires frame rows without padding and 16-byte aligned frame and state
+// planes. A bulk copy moves whole 16 bytes, four pixels of the frame: up to
+// three last pixels of an image come by plain loads. copy_frame = false leaves the frame segment to the
 // consumers (they foveate the frame into it themselves).
 template <int T>
 __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const FrameDev& f, int K,
@@ -91,14 +92,14 @@ __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const Fram
                                                   uint32_t stage_cap = 0xFFFFFFFFu) {
   const int64_t rem_plane = s.plane - p0, rem_px = s.hw - p0;
   const uint32_t n = static_cast<uint32_t>(rem_plane < T ? rem_plane : T);  // plane entries (x64)
-  const uint32_t np = static_cast<uint32_t>(rem_px < T ? rem_px : T);       // pixels (x4)
+  const uint32_t np = static_cast<uint32_t>(rem_px < T ? rem_px : T);       // pixels
 #ifdef WRS_CHECKED
   // every copy's global range inside its plane or the frame, and the stage's
   // layout inside the ring's stage; otherwise no copy is issued and the
   // barrier completes empty (the consumers then compute stale data, flagged)
   {
     bool ok = WRS_IN(s, p0 >= 0 && p0 < s.hw && p0 + n <= s.plane && p0 + np <= s.hw &&
-                            n % 64 == 0 && np % 4 == 0 && K >= 1 && K <= WRS_MAX_K,
+                            n % 64 == 0 && K >= 1 && K <= WRS_MAX_K,
                      kChkCopy);
     ok = WRS_IN(s, L.bytes <= stage_cap, kChkStageSize) && ok;
     if (!ok) {
@@ -110,11 +111,17 @@ __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const Fram
 #else
   (void)stage_cap;
 #endif
+  const uint32_t np4 = np & ~3u;
+  if (copy_frame && np4 != np) {
+    if (static_cast<uint32_t>(lane) < 3u * (np - np4))
+      reinterpret_cast<float*>(stage + L.frame)[3u * np4 + lane] = f.frame[3 * (p0 + np4) + lane];
+    __syncwarp();
+  }
   // the literal rule (K = 1) reads no P and no key plane: copies 2 and 3 are skipped
   const int skip = s.literal ? 2 : 0;
   const int ncopy = 3 + K + (resolve ? (cs == 2 ? 2 * K : K) : 0);
   if (lane == 0) {
-    uint32_t bytes = (copy_frame ? 12u * np : 0u) + 8u * n + 4u * K * n;
+    uint32_t bytes = (copy_frame ? 12u * np4 : 0u) + 8u * n + 4u * K * n;
     if (skip) bytes -= 4u * n + 4u * K * n;
     if (resolve) bytes += cs == 2 ? (2u * K * n + 8u * K * n) : 16u * K * n;
     mbar_arrive_expect_tx(bar, bytes + extra_tx);
@@ -123,9 +130,9 @@ __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const Fram
   const int64_t pl = s.plane;
   for (int c = lane; c < ncopy; c += 32) {
     if (skip && (c == 2 || c == 3)) continue;
-    if (c == 0 && !copy_frame) continue;
+    if (c == 0 && (!copy_frame || np4 == 0u)) continue;
     if (c == 0) {
-      bulk_g2s(stage + L.frame, f.frame + 3 * p0, 12u * np, bar);
+      bulk_g2s(stage + L.frame, f.frame + 3 * p0, 12u * np4, bar);
     } else if (c == 1) {
       bulk_g2s(stage + L.W, s.W + p0, 4u * n, bar);
     } else if (c == 2) {

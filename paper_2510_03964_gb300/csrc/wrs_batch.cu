@@ -181,7 +181,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
         return rc;
     } else {
       fr = d_frames[i];
-      if (!fr || !wrs_pipe_supported(x, fr, 3 * static_cast<int64_t>(x->cfg.width), out))
+      if (!fr || x->cfg.width % 4 != 0 || !wrs_pipe_supported(x, fr, 3 * static_cast<int64_t>(x->cfg.width), out))
         return wrs_fail(WRS_ERR_ARG,
                         "stream %d: batched frames need width %% 4 == 0 and 16-byte aligned, "
                         "unpadded frame and out",

@@ -457,7 +457,12 @@ extern "C" int wrs_push_frame(wrs_ctx* x, const float* d_frame, int64_t pitch, f
   f.map_lo = wrs_map_lo(x);
   cudaError_t e;
   if (x->pipe && wrs_pipe_supported(x, d_frame, pitch, d_out)) {
-    e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, x->pipe_px, x->pipe_stages, x->pipe_ctas,
+    int px = x->pipe_px, stages = x->pipe_stages;
+    if (px != 1 && x->cfg.width % 4 != 0) {
+      px = 1;  // a thread's pixels lie in one row: see wrs_pipe_supported
+      stages = wrs_default_stages(x->cfg.K, x->cfg.color_fp16 != 0, 1);
+    }
+    e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, px, stages, x->pipe_ctas,
                         wrs_status_word(x), x->timeout_ns, x->test_extra_tx,
                         static_cast<cudaStream_t>(stream));
   } else {

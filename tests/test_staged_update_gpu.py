@@ -48,3 +48,26 @@ def test_rare_branches_equal_the_plain_kernel(K, rule, fp16, bias, out):
     assert np.array_equal(a.export_raw()[256:], b.export_raw()[256:])
     assert a.replacements() == b.replacements()
     assert torch.equal(outs[0].view(torch.int32), outs[1].view(torch.int32))
+
+
+@pytest.mark.parametrize("K,rule,fp16", [(1, 1, False), (2, 0, True), (4, 0, False), (5, 0, True), (8, 0, False)])
+@pytest.mark.parametrize("wh", [(1, 1), (3, 1), (1, 7), (255, 1), (257, 1), (259, 3), (85, 6), (1365, 96), (134, 33)])
+def test_any_width_equals_the_plain_kernel(wh, K, rule, fp16):
+    """Widths not divisible by 4 (every remainder of the last tile and of the
+    frame's last 16 bytes) through the pipelined kernel."""
+    w, h = wh
+    rng = np.random.default_rng(w + h)
+    a, b = (wrs.Stream(w, h, K, 20.0, seed=6, color_fp16=fp16, update_rule=rule) for _ in range(2))
+    b.set_pipeline(False)
+    outs = [torch.full((h, w, 3), -1.0, device="cuda") for _ in range(2)]
+    for t in range(18):
+        frame = torch.from_numpy(rng.random((h, w, 3), dtype=np.float32)).cuda()
+        fm = torch.from_numpy(rng.choice(np.uint8([0, 255]), (h, w), p=[0.9, 0.1])).cuda() if t % 4 == 3 else None
+        for st, o in zip((a, b), outs):
+            st.push_frame(frame, (0.4 * w, 0.6 * h), fov_map=fm, out=o)
+    assert a.check_status() == 0
+    x, y = a.export_state(), b.export_state()
+    for plane in x:
+        assert np.array_equal(x[plane].view(np.uint8), y[plane].view(np.uint8)), plane
+    assert a.replacements() == b.replacements()
+    assert torch.equal(outs[0].view(torch.int32), outs[1].view(torch.int32))
