@@ -2,13 +2,11 @@
 // mip-mapped and each ring around the gaze is reconstructed from a coarser
 // level, by nearest lookup or bilinear filtering. Two kernels:
 //
-//  mip_kernel     one pass over the image builds every stored level. A CTA
-//                 stages a 2^M-row strip of 2048 pixels in shared memory
-//                 (M = top level), then forms the level sums bottom-up in
-//                 shared memory with the quad-tree order (s00 + s01) +
-//                 (s10 + s11) and writes each level's means as 16-byte
-//                 texels. The image is read once; levels >= 1 are written
-//                 once.
+//  mip_kernel     one pass over the image builds every stored level: the level
+//                 sums are formed bottom-up in registers with the quad-tree
+//                 order (s00 + s01) + (s10 + s11) and each level's means are
+//                 written as 16-byte texels. The image is read once; levels
+//                 >= 1 are written once.
 //  foveate4_kernel four adjacent pixels per thread (foveate_kernel: one, for
 //                 widths not divisible by 4 or unaligned frames): FP32 ring
 //                 test, then a copy of the image pixel (level 0) or one (box)
@@ -31,8 +29,9 @@ using wrs::MipLevelDev;
 namespace {
 
 constexpr int kMipThreads = 256;
-constexpr int kTilePx = 2048;          // pixels per CTA strip: 2^M rows x (2048 >> M) columns
+constexpr int kMipTileW = 64, kMipTileH = 32;  // pixels per CTA
 constexpr int kFovThreads = 256;
+constexpr int kFovTileW = 64, kFovTileH = 16;  // pixels per CTA of the four-pixel form
 
 // Writable view of a stored level, for the build.
 struct MipLevelOut {
@@ -57,107 +56,129 @@ struct FovArgs {
   float gx, gy;
 };
 
+// Pixels of level-L block i along an axis of n pixels.
 __device__ __forceinline__ int32_t block_extent(int32_t n, int32_t i, int L) {
   const int64_t lo = (int64_t)i << L;
   const int64_t hi = lo + ((int64_t)1 << L);
   return (int32_t)((hi < n ? hi : n) - lo);
 }
 
-// Shared memory of one strip: the pixels, then the sums of levels 1..M.
-// Level L of the strip holds (2^M >> L) rows x ((2048 >> M) >> L) texels x 3.
+// Writes texel (x, y) of level L from its block's sums, if the level has it.
+// A whole block's count is a power of two: its division is a multiplication.
+template <int L>
+__device__ __forceinline__ void store_mean(const MipArgs& a, uint32_t x, int32_t y, const float (&sum)[3]) {
+  const MipLevelOut& lv = a.lev[L];
+  if (x >= (uint32_t)lv.wb || y >= lv.hb) return;
+  float4 m;
+  if (((x + 1) << L) <= (uint32_t)a.width && ((y + 1) << L) <= a.height) {
+    constexpr float inv = 1.0f / (1 << (2 * L));
+    m = make_float4(__fmul_rn(sum[0], inv), __fmul_rn(sum[1], inv), __fmul_rn(sum[2], inv), 0.0f);
+  } else {
+    const float n = (float)(block_extent(a.height, y, L) * block_extent(a.width, (int32_t)x, L));
+    m = make_float4(__fdiv_rn(sum[0], n), __fdiv_rn(sum[1], n), __fdiv_rn(sum[2], n), 0.0f);
+  }
+  lv.texels[(int64_t)y * lv.wb + x] = m;
+}
+
+// A CTA builds every level of a 64 x 32 pixel tile: eight warps of 32 x 8
+// pixels, a lane four pixels of two rows. A lane's registers hold its pixels,
+// its two level-1 sums and, after one exchange per axis (shuffles), the sums of
+// levels 2 and 3; only levels 4 and 5 meet in shared memory. Sums are the
+// quad-tree order's, (s00 + s01) + (s10 + s11). Bound by DRAM and the L2: the
+// form that staged the strip in shared memory waited on its barriers and
+// strided reads, 26.7 us for a 4K image's three levels; this one 21.
 template <int M, bool VEC>
 __global__ void __launch_bounds__(kMipThreads) mip_kernel(MipArgs a) {
-  constexpr int TH = 1 << M;
-  constexpr int TW = kTilePx >> M;
-  constexpr int kRowF = TW * 3;
-  __shared__ __align__(16) float s_px[kTilePx * 3];
-  // levels 1..M of a strip hold sum_L 2048 / 4^L < 2048 / 3 texels
-  __shared__ float s_sum[(kTilePx / 3 + 1) * 3];
+  __shared__ float s_sum[4][8][3];  // level-3 sums of the tile (M > 3)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rp = lane >> 3, cq = lane & 7;  // row pair and column quad in the warp's 8 x 32
+  wrs::grid_begin();
+  const uint32_t x0 = blockIdx.x * kMipTileW + (warp & 1) * 32 + 4 * cq;
+  const int32_t y0 = blockIdx.y * kMipTileH + (warp >> 1) * 8 + 2 * rp;
+  // pixels from x0 to the end of the row (none past it)
+  const int32_t left = (int32_t)((uint32_t)a.width - x0);
 
-  const int tid = threadIdx.x;
-  const int64_t ty0 = (int64_t)blockIdx.y * TH;
-  const int64_t tx0 = (int64_t)blockIdx.x * TW;
-  const int64_t row_f = 3 * (int64_t)a.width;
-
-  // stage the strip (zero outside the image), coalesced along each row
-  if (VEC) {
-    // 16-byte loads: rows start 16-byte aligned (pitch % 4 == 0, tx0 % 4 == 0);
-    // all of a thread's loads are issued before any is stored to shared memory
-    constexpr int kRowQ = kRowF / 4;
-    constexpr int kPer = kTilePx * 3 / 4 / kMipThreads;
-    float4 v[kPer];
+  float v[2][12];
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      const int q = tid + j * kMipThreads;
-      const int r = q / kRowQ, c4 = q - r * kRowQ;
-      const int64_t y = ty0 + r;
-      const int64_t lim = y < a.height ? row_f - 3 * tx0 : 0;
-      const float* src = a.img + (y < a.height ? y : 0) * a.pitch + 3 * tx0 + 4 * c4;
-      const int64_t f0 = 4 * (int64_t)c4;
-      if (f0 + 4 <= lim) {
-        v[j] = __ldg(reinterpret_cast<const float4*>(src));
-      } else {
-        v[j].x = f0 < lim ? __ldg(src) : 0.0f;
-        v[j].y = f0 + 1 < lim ? __ldg(src + 1) : 0.0f;
-        v[j].z = f0 + 2 < lim ? __ldg(src + 2) : 0.0f;
-        v[j].w = 0.0f;
+  for (int r = 0; r < 2; ++r) {
+    const int32_t y = y0 + r;
+    const float* src = a.img + (int64_t)y * a.pitch + 3 * (int64_t)x0;
+    if (VEC && y < a.height && left >= 4) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const float4 t = __ldg(reinterpret_cast<const float4*>(src) + i);
+        v[r][4 * i] = t.x;
+        v[r][4 * i + 1] = t.y;
+        v[r][4 * i + 2] = t.z;
+        v[r][4 * i + 3] = t.w;
       }
-    }
+    } else {
+      // pixels outside the image count as 0
+      const int in_row = y < a.height ? 3 * (left < 4 ? left : 4) : 0;
 #pragma unroll
-    for (int j = 0; j < kPer; ++j)
-      reinterpret_cast<float4*>(s_px)[tid + j * kMipThreads] = v[j];
-  } else {
-    for (int r = 0; r < TH; ++r) {
-      const int64_t y = ty0 + r;
-      // floats of this row inside the image (none below the last row)
-      const int64_t lim = y < a.height ? row_f - 3 * tx0 : 0;
-      const float* src = a.img + (y < a.height ? y : 0) * a.pitch + 3 * tx0;
-      for (int i = tid; i < kRowF; i += kMipThreads)
-        s_px[r * kRowF + i] = i < lim ? __ldg(src + i) : 0.0f;
+      for (int i = 0; i < 12; ++i) v[r][i] = i < in_row ? __ldg(src + i) : 0.0f;
     }
   }
-  __syncthreads();
 
-  // level L sums from level L-1 (level 0 = the staged pixels)
-  const float* prev = s_px;
-  int prev_w = TW;
-  float* cur = s_sum;
+  float s[2][3];
 #pragma unroll
-  for (int L = 1; L <= M; ++L) {
-    const int lw = TW >> L;
-    const int lh = TH >> L;
-    const int n = lw * lh;
-    const MipLevelOut lv = a.lev[L];
-    for (int i = tid; i < n; i += kMipThreads) {
-      const int r = i / lw, c = i - r * lw;
-      const float* p0 = prev + ((2 * r) * prev_w + 2 * c) * 3;
-      const float* p1 = p0 + prev_w * 3;
-      float s[3];
+  for (int c = 0; c < 2; ++c) {
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch)
+      s[c][ch] = __fadd_rn(__fadd_rn(v[0][6 * c + ch], v[0][6 * c + 3 + ch]),
+                           __fadd_rn(v[1][6 * c + ch], v[1][6 * c + 3 + ch]));
+    store_mean<1>(a, (x0 >> 1) + c, y0 >> 1, s[c]);
+  }
+  if constexpr (M >= 2) {
+    float t[3];
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) {
+      t[ch] = __fadd_rn(s[0][ch], s[1][ch]);
+      t[ch] = __fadd_rn(t[ch], __shfl_xor_sync(0xffffffffu, t[ch], 8));
+    }
+    if ((rp & 1) == 0) store_mean<2>(a, x0 >> 2, y0 >> 2, t);
+    if constexpr (M >= 3) {
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) {
-        const float top = __fadd_rn(p0[ch], p0[3 + ch]);
-        const float bot = __fadd_rn(p1[ch], p1[3 + ch]);
-        s[ch] = __fadd_rn(top, bot);
-        cur[i * 3 + ch] = s[ch];
+        t[ch] = __fadd_rn(t[ch], __shfl_xor_sync(0xffffffffu, t[ch], 1));
+        t[ch] = __fadd_rn(t[ch], __shfl_xor_sync(0xffffffffu, t[ch], 16));
       }
-      const int32_t gy = (int32_t)(ty0 >> L) + r;
-      const int32_t gx = (int32_t)(tx0 >> L) + c;
-      if (gy < lv.hb && gx < lv.wb) {
-        const float cnt = (float)(block_extent(a.height, gy, L) * block_extent(a.width, gx, L));
-        lv.texels[(int64_t)gy * lv.wb + gx] =
-            make_float4(__fdiv_rn(s[0], cnt), __fdiv_rn(s[1], cnt), __fdiv_rn(s[2], cnt), 0.0f);
+      const bool top = rp == 0 && (cq & 1) == 0;
+      if (top) store_mean<3>(a, x0 >> 3, y0 >> 3, t);
+      if constexpr (M >= 4) {
+        if (top) {
+#pragma unroll
+          for (int ch = 0; ch < 3; ++ch) s_sum[warp >> 1][(warp & 1) * 4 + (cq >> 1)][ch] = t[ch];
+        }
+        __syncthreads();
+        if (warp == 0) {
+          // lanes 0..7: the tile's 2 x 4 level-4 texels, then 1 x 2 of level 5
+          const int r = (lane >> 2) & 1, c = lane & 3;
+#pragma unroll
+          for (int ch = 0; ch < 3; ++ch)
+            t[ch] = __fadd_rn(__fadd_rn(s_sum[2 * r][2 * c][ch], s_sum[2 * r][2 * c + 1][ch]),
+                              __fadd_rn(s_sum[2 * r + 1][2 * c][ch], s_sum[2 * r + 1][2 * c + 1][ch]));
+          const uint32_t gx = blockIdx.x * (kMipTileW >> 4) + c;
+          const int32_t gy = blockIdx.y * (kMipTileH >> 4) + r;
+          if (lane < 8) store_mean<4>(a, gx, gy, t);
+          if constexpr (M >= 5) {
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) {
+              t[ch] = __fadd_rn(t[ch], __shfl_xor_sync(0xffffffffu, t[ch], 1));
+              t[ch] = __fadd_rn(t[ch], __shfl_xor_sync(0xffffffffu, t[ch], 4));
+            }
+            if (lane < 4 && (lane & 1) == 0) store_mean<5>(a, gx >> 1, gy >> 1, t);
+          }
+        }
       }
     }
-    __syncthreads();
-    prev = cur;
-    prev_w = lw;
-    cur += n * 3;
   }
 }
 
 // One pixel per thread (any width, pitch and alignment).
 template <int FILTER>
 __global__ void __launch_bounds__(kFovThreads) foveate_kernel(FovArgs a) {
+  wrs::grid_begin();
   const int64_t n = (int64_t)a.width * a.height;
   for (int64_t p = (int64_t)blockIdx.x * kFovThreads + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * kFovThreads) {
@@ -178,12 +199,18 @@ __global__ void __launch_bounds__(kFovThreads) foveate_kernel(FovArgs a) {
 // its 48 bytes of colour as three 16-byte stores and its levels as one word.
 template <int FILTER>
 __global__ void __launch_bounds__(kFovThreads) foveate4_kernel(FovArgs a) {
-  const int32_t wq = a.width >> 2;
-  const int64_t nq = (int64_t)wq * a.height;
-  for (int64_t q = (int64_t)blockIdx.x * kFovThreads + threadIdx.x; q < nq;
-       q += (int64_t)gridDim.x * kFovThreads) {
-    const int32_t y = (int32_t)(q / wq);
-    const int32_t x0 = 4 * (int32_t)(q - (int64_t)y * wq);
+  // a warp takes 8 quads of 4 rows (32 x 4 pixels) and a CTA 2 x 4 warps
+  // (64 x 16): fewer warps straddle a ring's border, where a warp runs the code
+  // of both levels, than with 32 quads of one row
+  wrs::grid_begin();
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t tiles_x = ((uint32_t)a.width + kFovTileW - 1) / kFovTileW;
+  const uint32_t tiles = tiles_x * (((uint32_t)a.height + kFovTileH - 1) / kFovTileH);
+  for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const uint32_t ty = t / tiles_x;
+    const int32_t x0 = (int32_t)((t - ty * tiles_x) * kFovTileW + (warp & 1) * 32 + 4 * (lane & 7));
+    const int32_t y = (int32_t)(ty * kFovTileH + (warp >> 1) * 4 + (lane >> 3));
+    if (x0 >= a.width || y >= a.height) continue;
     float rgb[12];
     const uint32_t lv = wrs::fov_quad<FILTER>(a.fv, a.gx, a.gy, x0, y, rgb);
     float4* o = reinterpret_cast<float4*>(a.frame + (int64_t)y * a.frame_pitch + 3 * (int64_t)x0);
@@ -268,14 +295,16 @@ extern "C" int wrs_mip_build(const float* d_img, int64_t pitch, int32_t width, i
   a.top = levels - 1;
   fill_levels(L, d_mip, a.lev);
   const int M = levels - 1;
-  const int TH = 1 << M, TW = kTilePx >> M;
-  const dim3 grid((unsigned)((width + TW - 1) / TW), (unsigned)((height + TH - 1) / TH));
-  if (grid.y > 65535u) return wrs_fail(WRS_ERR_ARG, "image too tall for the mip build");
+  const dim3 grid((unsigned)(((int64_t)width + kMipTileW - 1) / kMipTileW),
+                  (unsigned)(((int64_t)height + kMipTileH - 1) / kMipTileH));
+  if ((((int64_t)height + (1 << M) - 1) >> M) > 65535)
+    return wrs_fail(WRS_ERR_ARG, "image too tall for the mip build");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool vec = pitch % 4 == 0 && aligned(d_img, 16);
-#define WRS_MIP_LAUNCH(m)                                                   \
-  (vec ? mip_kernel<m, true><<<grid, kMipThreads, 0, st>>>(a)               \
-       : mip_kernel<m, false><<<grid, kMipThreads, 0, st>>>(a))
+  cudaError_t e;
+#define WRS_MIP_LAUNCH(m)                                                    \
+  (e = vec ? wrs_launch_early(mip_kernel<m, true>, grid, kMipThreads, 0, st, a) \
+           : wrs_launch_early(mip_kernel<m, false>, grid, kMipThreads, 0, st, a))
   switch (M) {
     case 1: WRS_MIP_LAUNCH(1); break;
     case 2: WRS_MIP_LAUNCH(2); break;
@@ -284,7 +313,6 @@ extern "C" int wrs_mip_build(const float* d_img, int64_t pitch, int32_t width, i
     default: WRS_MIP_LAUNCH(5); break;
   }
 #undef WRS_MIP_LAUNCH
-  cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? WRS_OK : wrs_cuda_fail(e, "wrs_mip_build: launch");
 }
 
@@ -346,21 +374,16 @@ extern "C" int wrs_foveate(const float* d_img, int64_t pitch, const void* d_mip,
   if (int rc = device_sms(&sms)) return rc;
   const bool quad = width % 4 == 0 && frame_pitch % 4 == 0 && aligned(d_frame, 16) &&
                     (!d_ring || aligned(d_ring, 4));
-  const int64_t n = (int64_t)width * height / (quad ? 4 : 1);
-  const int64_t want = (n + kFovThreads - 1) / kFovThreads;
+  const int64_t want = quad ? (((int64_t)width + kFovTileW - 1) / kFovTileW) *
+                                  (((int64_t)height + kFovTileH - 1) / kFovTileH)
+                            : ((int64_t)width * height + kFovThreads - 1) / kFovThreads;
   const int64_t cap = (int64_t)sms * 8 * 16;  // 8 resident CTAs per SM x 16 waves
   const unsigned grid = (unsigned)(want < cap ? want : cap);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (quad) {
-    if (filter == WRS_FILTER_BOX)
-      foveate4_kernel<WRS_FILTER_BOX><<<grid, kFovThreads, 0, st>>>(a);
-    else
-      foveate4_kernel<WRS_FILTER_BILINEAR><<<grid, kFovThreads, 0, st>>>(a);
-  } else if (filter == WRS_FILTER_BOX) {
-    foveate_kernel<WRS_FILTER_BOX><<<grid, kFovThreads, 0, st>>>(a);
-  } else {
-    foveate_kernel<WRS_FILTER_BILINEAR><<<grid, kFovThreads, 0, st>>>(a);
-  }
-  cudaError_t e = cudaGetLastError();
+  const auto kernel = quad ? (filter == WRS_FILTER_BOX ? foveate4_kernel<WRS_FILTER_BOX>
+                                                       : foveate4_kernel<WRS_FILTER_BILINEAR>)
+                           : (filter == WRS_FILTER_BOX ? foveate_kernel<WRS_FILTER_BOX>
+                                                       : foveate_kernel<WRS_FILTER_BILINEAR>);
+  const cudaError_t e = wrs_launch_early(kernel, dim3(grid), kFovThreads, 0, st, a);
   return e == cudaSuccess ? WRS_OK : wrs_cuda_fail(e, "wrs_foveate: launch");
 }

@@ -35,6 +35,24 @@ constexpr int kDefaultPx = 4;
 constexpr uint64_t kDefaultTimeoutNs = 2000000000ull;  // 2 s
 constexpr size_t kSmemBudget = 227 * 1024 - 1024;       // dynamic shared memory per CTA we use
 
+// Launches a kernel that calls wrs::grid_begin: it may start before the
+// previous kernel of the stream has ended.
+template <typename... P, typename... A>
+cudaError_t wrs_launch_early(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                             cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t how = {};
+  how.gridDim = grid;
+  how.blockDim = dim3(threads);
+  how.dynamicSmemBytes = smem;
+  how.stream = st;
+  how.attrs = &early;
+  how.numAttrs = 1;
+  return cudaLaunchKernelEx(&how, kernel, args...);
+}
+
 uint32_t* wrs_status_word(const wrs_ctx* x);
 size_t wrs_pipe_smem_bytes(int K, bool f16, int px, int stages, bool resolve);
 bool wrs_pipe_supported(const wrs_ctx* x, const float* frame, int64_t pitch, const float* out);
