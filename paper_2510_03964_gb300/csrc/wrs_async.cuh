@@ -176,12 +176,14 @@ __device__ __forceinline__ void draw_tile_uniforms(const StreamDev& s, const Fra
 }
 
 // What a consumer thread of a tile knows before the tile has landed: its first
-// pixel p = (x, y) (no pixel if p >= hw), the flush bits of its PX pixels and,
-// in the band this frame folds, the fold's inputs. Loaded ahead of the wait,
-// so that their latency passes while the tile is still in flight.
+// pixel p = (x, y) (no pixel if p >= hw), the flush-map entries of its PX
+// pixels and, in the band this frame folds, the fold's inputs. Loaded ahead of
+// the wait and first used after it, so that their latency passes while the
+// tile is still in flight.
 template <int KM>
 struct TilePx {
-  uint32_t p, flush;
+  uint32_t p;
+  uint32_t fov[4];  // the pixels' flush-map entries
   int x, y;
   bool folding;
   FoldIn<KM> fold;
@@ -190,10 +192,14 @@ struct TilePx {
 // Fills t for the pixels at t.p (t.x and t.y already set).
 template <int KM, int PX, bool FOLD>
 __device__ __forceinline__ void tile_ahead(const StreamDev& s, const FrameDev& f, TilePx<KM>& t) {
-  t.flush = 0;
+#pragma unroll
+  for (int i = 0; i < PX; ++i) t.fov[i] = 0u;
   t.folding = false;
   if (t.p >= static_cast<uint32_t>(s.hw)) return;
-  t.flush = flush_bits<PX>(f, t.p);
+  if (f.fov != nullptr) {
+#pragma unroll
+    for (int i = 0; i < PX; ++i) t.fov[i] = f.fov[static_cast<int64_t>(t.p) + i];
+  }
   if constexpr (FOLD && PX == 1) {
     if (s.K > 2 && s.K <= KM && folds_now(f, t.p)) {
       fold_load(s, s.idx, s.K, f.t, t.p, t.fold);
@@ -204,24 +210,44 @@ __device__ __forceinline__ void tile_ahead(const StreamDev& s, const FrameDev& f
 
 // Computes consumer thread `tid`'s PX pixels of a landed tile from shared
 // memory; returns how many of them replaced a slot. LIT: the literal n = 1
-// rule (KT = 1). FILTER >= 0: the thread first foveates its pixels of the
-// frame from `fv` into the stage's frame segment (the producer copied no
-// frame); each thread writes and then reads only its own pixels there.
-template <int KT, bool F16, int PX, int T, bool LIT, int FILTER, int KM>
-__device__ __forceinline__ int compute_tile(const StreamDev& s, const FrameDev& f, const FovDev& fv,
-                                            uint8_t* st, const float* u, const TilePx<KM>& t,
-                                            float d_f, int tid) {
+// rule (KT = 1).
+template <int KT, bool F16, int PX, int T, bool LIT, int KM>
+__device__ __forceinline__ int compute_tile(const StreamDev& s, const FrameDev& f, uint8_t* st,
+                                            const float* u, const TilePx<KM>& t, float d_f, int tid) {
   if (t.p >= static_cast<uint32_t>(s.hw)) return 0;
-  if constexpr (FILTER >= 0) {
-    float* fr = reinterpret_cast<float*>(st) + 3 * tid * PX;
+  uint32_t flush = 0;
 #pragma unroll
-    for (int i = 0; i < PX; ++i) fov_pixel<FILTER>(fv, f.gx, f.gy, t.x + i, t.y, fr + 3 * i);
-  }
+  for (int i = 0; i < PX; ++i) flush |= t.fov[i] == 0xFFu ? 1u << i : 0u;
   if constexpr (LIT)
-    return push_staged_literal<F16, PX, T>(s, f, st, u, t.p, t.x, t.y, d_f, tid, t.flush);
+    return push_staged_literal<F16, PX, T>(s, f, st, u, t.p, t.x, t.y, d_f, tid, flush);
   else
-    return push_staged<KT, F16, PX, T, KM>(s, f, st, u, t.p, t.x, t.y, d_f, tid, t.flush,
+    return push_staged<KT, F16, PX, T, KM>(s, f, st, u, t.p, t.x, t.y, d_f, tid, flush,
                                            t.folding ? &t.fold : nullptr);
+}
+
+// Frames foveated on read: two warps (w = 0, 1) write the 256-pixel tile's
+// foveated colours into the stage's frame segment, four pixels per lane, and
+// arrive on `bar`. With the consumers foveating their own pixels one by one, a
+// 4K K = 8 FP16 frame (mip levels and update) takes 261 us instead of 259.
+constexpr int kFovWarps = 2;
+template <int FILTER>
+__device__ __forceinline__ void foveate_tile(const StreamDev& s, const FrameDev& f, const FovDev& fv,
+                                             uint32_t tile, uint8_t* stage, uint64_t* bar, int w,
+                                             int lane) {
+  const uint32_t q = 4u * (32u * w + lane);  // the lane's first pixel in the tile
+  const uint32_t p = tile * 256u + q;
+  if (p < static_cast<uint32_t>(s.hw)) {
+    int y, x;
+    row_col(s, static_cast<int>(p), y, x);
+    float rgb[12];
+    fov_quad<FILTER>(fv, f.gx, f.gy, x, y, rgb);
+    float4* o = reinterpret_cast<float4*>(stage) + 3 * (q / 4);
+    o[0] = make_float4(rgb[0], rgb[1], rgb[2], rgb[3]);
+    o[1] = make_float4(rgb[4], rgb[5], rgb[6], rgb[7]);
+    o[2] = make_float4(rgb[8], rgb[9], rgb[10], rgb[11]);
+  }
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar);
 }
 
 // Adds a warp's counts to a running total: one atomic per warp.
@@ -286,6 +312,7 @@ struct Ring {
   uint32_t stage_bytes;  // planes of the largest tile layout used
   uint32_t stride;       // stage_bytes + 4 * T
   int S;
+  bool queue;            // the grid has more tiles than CTAs that fit: ask for more
   uint64_t* full;
   uint64_t* empty;
   uint64_t* told;        // [kAnswers]
@@ -300,8 +327,10 @@ __host__ __device__ __forceinline__ size_t ring_bytes(uint32_t stage_bytes, int 
   return static_cast<size_t>(S) * (stage_bytes + 4u * T) + 16u * S + 24u * kAnswers + 16u;
 }
 
-__device__ __forceinline__ Ring make_ring(uint8_t* smem, uint32_t stage_bytes, int T, int S) {
+__device__ __forceinline__ Ring make_ring(uint8_t* smem, uint32_t stage_bytes, int T, int S,
+                                          bool queue) {
   Ring r;
+  r.queue = queue;
   r.base = smem;
   r.stage_bytes = stage_bytes;
   r.stride = stage_bytes + 4u * T;
@@ -314,16 +343,16 @@ __device__ __forceinline__ Ring make_ring(uint8_t* smem, uint32_t stage_bytes, i
   return r;
 }
 
-// Thread 0 initialises the barriers (full: two arrivals, the copying warp's
-// and the drawing warp's; empty: one arrival per consumer warp; told: the
+// One warp initialises the barriers (full: one arrival per producing warp, the
+// copying, the drawing and any foveating ones; empty: one arrival per consumer warp; told: the
 // request's) and the flag; the caller then synchronises the block.
-__device__ __forceinline__ void init_ring(const Ring& r, int consumer_warps) {
-  for (int i = 0; i < r.S; ++i) {
-    mbar_init(&r.full[i], 2);
-    mbar_init(&r.empty[i], consumer_warps);
+__device__ __forceinline__ void init_ring(const Ring& r, int consumer_warps, int producer_warps, int lane) {
+  if (lane < r.S) {
+    mbar_init(&r.full[lane], producer_warps);
+    mbar_init(&r.empty[lane], consumer_warps);
   }
-  for (int i = 0; i < kAnswers; ++i) mbar_init(&r.told[i], 1);
-  *r.flag = 0;
+  if (lane < kAnswers) mbar_init(&r.told[lane], 1);
+  if (lane == 0) *r.flag = 0;
   fence_mbar_init();
 }
 
@@ -345,6 +374,7 @@ struct TileWalk {
 
   // Moves to the next tile; false when there is none or the wait gave up.
   __device__ __forceinline__ bool next(const Ring& r, uint64_t timeout_ns) {
+    if (!r.queue) return false;
     if (!mbar_wait_bounded(&r.told[slot], phase, timeout_ns)) {
       raise_flag(r);
       return false;
@@ -360,7 +390,7 @@ struct TileWalk {
 
 // A producer warp: for each of the CTA's tiles, waits until the stage is free
 // and runs `tile_fn(tile, stage, u, full_bar, lane)`, which issues the tile's
-// copies (the copying warp) or draws its uniforms (the drawing warp) and
+// copies (the copying warp), draws its uniforms or foveates its frame, and
 // arrives on the stage's full barrier. The copying warp (ASK) also asks for
 // the tiles, one ahead of the one it copies: the answer it overwrites is that
 // of a tile whose stage has since been freed. Returns the number of tiles
@@ -370,7 +400,7 @@ __device__ __forceinline__ int produce(const Ring& r, uint64_t timeout_ns, int l
   TileWalk at(blockIdx.x);
   int it = 0, stg = 0, ask = 0;
   uint32_t phase = 1;  // of the stage's last release; the first S tiles wait for none
-  if (ASK && lane == 0) request_tile(&r.answer[0], &r.told[0]);
+  if (ASK && r.queue && lane == 0) request_tile(&r.answer[0], &r.told[0]);
   do {
     if (it >= r.S && !mbar_wait_bounded(&r.empty[stg], phase, timeout_ns)) {
       raise_flag(r);
@@ -391,7 +421,7 @@ __device__ __forceinline__ int produce(const Ring& r, uint64_t timeout_ns, int l
     }
   } while (true);
   // a wait gave up: an answer still on its way lands before the CTA may end
-  if (ASK && flag_raised(r)) mbar_wait_bounded(&r.told[at.slot], at.phase, timeout_ns);
+  if (ASK && r.queue && flag_raised(r)) mbar_wait_bounded(&r.told[at.slot], at.phase, timeout_ns);
   return it;
 }
 

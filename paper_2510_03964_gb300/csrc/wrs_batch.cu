@@ -254,18 +254,22 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     b->configured_smem[slot] = kSmemBudget;
   }
   int fit = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, fn, kBatchThreads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, fn, batch_threads(fov), smem);
   if (e != cudaSuccess) return wrs_cuda_fail(e, "push_batch: occupancy");
   if (fit < 1) return wrs_fail(WRS_ERR_ARG, "batch kernel does not fit on an SM");
   // fewer CTAs per SM than fit: a larger shared-memory request keeps the others out
-  if (b->ctas_per_sm > 0 && b->ctas_per_sm < fit) smem = wrs::smem_for_ctas(smem, b->ctas_per_sm);
+  if (b->ctas_per_sm > 0 && b->ctas_per_sm < fit) {
+    smem = wrs::smem_for_ctas(smem, b->ctas_per_sm);
+    fit = b->ctas_per_sm;
+  }
+  a.queue = tiles > static_cast<int64_t>(ctxs[0]->sms) * fit ? 1 : 0;
 
   cudaKernelNodeParams kp;
   std::memset(&kp, 0, sizeof kp);
   void* params[1] = {&a};
   kp.func = const_cast<void*>(fn);
   kp.gridDim = dim3(static_cast<unsigned>(tiles));  // one CTA per tile: see request_tile
-  kp.blockDim = dim3(kBatchThreads);
+  kp.blockDim = dim3(batch_threads(fov));
   kp.sharedMemBytes = static_cast<unsigned>(smem);
   kp.kernelParams = params;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);

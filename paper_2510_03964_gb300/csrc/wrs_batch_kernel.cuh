@@ -37,6 +37,7 @@ __device__ __forceinline__ bool stage_records(const BatchEntry& e) {
 
 struct BatchArgs {
   int n;
+  int queue;             // more tiles than CTAs that fit: see Ring::queue
   int stages;
   uint32_t stage_bytes;  // largest stage of any stream in the batch
   uint64_t timeout_ns;
@@ -59,7 +60,9 @@ __device__ __forceinline__ bool entry_f16(const BatchEntry& e) {
 }
 
 constexpr int kConsumerWarps = 8;
-constexpr int kBatchThreads = (kConsumerWarps + 2) * 32;
+// the copying and the drawing warp, and two that foveate frames on read
+constexpr int batch_producers(bool fov) { return fov ? 2 + wrs::kFovWarps : 2; }
+constexpr int batch_threads(bool fov) { return (kConsumerWarps + batch_producers(fov)) * 32; }
 
 // Adds a warp's running count of replacements in entry ei to the CTA's
 // per-stream total and clears it: once per stream a warp leaves, not per tile.
@@ -75,14 +78,13 @@ __device__ __forceinline__ void flush_count(unsigned long long* replaced_s, int 
 // holding only those two variants; any other mix gets the kernel with all.
 constexpr int kFamF16K48 = 0, kFamF32K48 = 1, kFamAll = 2;
 
-// One tile of entry e: the update from the staged frame, or (FOVF >= 0) from
-// the frame foveated on read. The fold inputs are held for up to 8 slots
+// One tile of entry e. The fold inputs are held for up to 8 slots
 // whatever the stream's K (no narrowed copy, which would have to live in local
 // memory); the generic-K and literal forms load their own.
-template <int KT, bool F16, int PX, int T, bool LIT, int FOVF>
+template <int KT, bool F16, int PX, int T, bool LIT>
 __device__ __forceinline__ int tile(const BatchEntry& e, uint8_t* st, const float* u,
                                     const wrs::TilePx<8>& px, float d_f, int tid) {
-  return wrs::compute_tile<KT, F16, PX, T, LIT, FOVF>(e.s, e.f, e.fv, st, u, px, d_f, tid);
+  return wrs::compute_tile<KT, F16, PX, T, LIT>(e.s, e.f, st, u, px, d_f, tid);
 }
 
 // The copying warp's work for one tile of entry e. KT, CS > 0 fix the slot count and colour bytes at compile time (the
@@ -99,10 +101,10 @@ __device__ __forceinline__ void produce_tile(const BatchEntry& e, int64_t p0, ui
 
 // Warp-specialised like the single-stream pipelined kernel: warp 8 issues each
 // tile's copies, warp 9 draws its uniforms, warps 0..7 compute it. FOVF >= 0:
-// no frame is copied; the consumers foveate each pixel from the stream's
-// image and mip levels (filter FOVF, WRS_FILTER_*) into the stage first.
+// no frame is copied; two more warps foveate each tile from the stream's
+// image and mip levels (filter FOVF, WRS_FILTER_*) into the stage.
 template <int PX, int FAM, int FOVF = -1>
-__global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
+__global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
     batch_kernel(const __grid_constant__ BatchArgs a) {
   static_assert(FOVF < 0 || PX == 1, "foveating batches take one pixel per thread");
   extern __shared__ __align__(128) uint8_t smem[];
@@ -110,11 +112,11 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
   __shared__ float d_f_s[kMaxBatch];                    // per stream: density at the fovea edge
   __shared__ uint32_t failed_s[kMaxBatch];              // per stream: an earlier wait gave up
   constexpr int T = kConsumerWarps * 32 * PX;
-  const wrs::Ring r = wrs::make_ring(smem, a.stage_bytes, T, a.stages);
+  const wrs::Ring r = wrs::make_ring(smem, a.stage_bytes, T, a.stages, a.queue != 0);
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
-  if (tid == 0) wrs::init_ring(r, kConsumerWarps);
+  if (warp == 0) wrs::init_ring(r, kConsumerWarps, batch_producers(FOVF >= 0), lane);
   if (tid < kMaxBatch) replaced_s[tid] = 0;
   // each stream's Eq. (phat) normaliser, once per CTA instead of once per tile
   if (tid < a.n) {
@@ -152,6 +154,15 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
       const BatchEntry& e = a.e[pe];
       wrs::draw_tile_uniforms<T>(e.s, e.f, static_cast<int64_t>(g - e.tile0) * T, u, full, ln);
     });
+  } else if (FOVF >= 0 && warp >= kConsumerWarps + 2) {
+    int pe = 0;
+    if constexpr (FOVF >= 0)
+      wrs::produce<false>(r, a.timeout_ns, lane,
+                          [&](uint32_t g, uint8_t* st, float*, uint64_t* full, int ln) {
+        pe = entry_after(a, g, pe);
+        const BatchEntry& e = a.e[pe];
+        wrs::foveate_tile<FOVF>(e.s, e.f, e.fv, g - e.tile0, st, full, warp - kConsumerWarps - 2, ln);
+      });
   } else {
     wrs::TilePx<8> px;
     int ei = 0;        // entry of the consumer's current tile
@@ -177,21 +188,21 @@ __global__ void __launch_bounds__(kBatchThreads, PX == 1 ? 2 : 1)
       if (failed_s[ei] != 0) return;
       int rc;
       if constexpr (FAM == kFamF16K48) {
-        rc = e.code == 0 ? tile<4, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid)
-                         : tile<8, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid);
+        rc = e.code == 0 ? tile<4, true, PX, T, false>(e, st, u, px, d_f, tid)
+                         : tile<8, true, PX, T, false>(e, st, u, px, d_f, tid);
       } else if constexpr (FAM == kFamF32K48) {
-        rc = e.code == 2 ? tile<4, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid)
-                         : tile<8, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid);
+        rc = e.code == 2 ? tile<4, false, PX, T, false>(e, st, u, px, d_f, tid)
+                         : tile<8, false, PX, T, false>(e, st, u, px, d_f, tid);
       } else {
         switch (e.code) {
-          case 0: rc = tile<4, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
-          case 1: rc = tile<8, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
-          case 2: rc = tile<4, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
-          case 3: rc = tile<8, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
-          case 4: rc = tile<0, true, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
-          case 6: rc = tile<1, true, PX, T, true, FOVF>(e, st, u, px, d_f, tid); break;
-          case 7: rc = tile<1, false, PX, T, true, FOVF>(e, st, u, px, d_f, tid); break;
-          default: rc = tile<0, false, PX, T, false, FOVF>(e, st, u, px, d_f, tid); break;
+          case 0: rc = tile<4, true, PX, T, false>(e, st, u, px, d_f, tid); break;
+          case 1: rc = tile<8, true, PX, T, false>(e, st, u, px, d_f, tid); break;
+          case 2: rc = tile<4, false, PX, T, false>(e, st, u, px, d_f, tid); break;
+          case 3: rc = tile<8, false, PX, T, false>(e, st, u, px, d_f, tid); break;
+          case 4: rc = tile<0, true, PX, T, false>(e, st, u, px, d_f, tid); break;
+          case 6: rc = tile<1, true, PX, T, true>(e, st, u, px, d_f, tid); break;
+          case 7: rc = tile<1, false, PX, T, true>(e, st, u, px, d_f, tid); break;
+          default: rc = tile<0, false, PX, T, false>(e, st, u, px, d_f, tid); break;
         }
       }
       replaced += rc;

@@ -510,18 +510,16 @@ __device__ __forceinline__ void fold_load(const StreamDev& s, const uint32_t* id
   const int64_t pl = s.plane;
 #pragma unroll
   for (int j = 0; j < KM; ++j) in.v[j] = j < K ? idx[j * pl + p] : kEmpty;
-  uint8_t b[kRingFrames];
+  uint32_t b[kRingFrames];
 #pragma unroll
   for (int k = 0; k < kRingFrames - 1; ++k) {
     const uint32_t fr = t - static_cast<uint32_t>(kRingFrames - 1) + k;
     b[k] = s.maps[static_cast<int64_t>(fr & kRingMask) * pl + p];
   }
-  b[kRingFrames - 1] = kCodeKeep;
+  b[kRingFrames - 1] = 0;  // this frame's: see fold_store
 #pragma unroll
   for (int w = 0; w < kRingFrames / 4; ++w)
-    in.code[w] = static_cast<uint32_t>(b[4 * w]) | (static_cast<uint32_t>(b[4 * w + 1]) << 8) |
-                 (static_cast<uint32_t>(b[4 * w + 2]) << 16) |
-                 (static_cast<uint32_t>(b[4 * w + 3]) << 24);
+    in.code[w] = b[4 * w] | (b[4 * w + 1] << 8) | (b[4 * w + 2] << 16) | (b[4 * w + 3] << 24);
 }
 
 // Left shifts that give 0 for amounts of 32 and above (and for negative ones).
@@ -535,9 +533,9 @@ __device__ __forceinline__ uint32_t shl_or_0(uint32_t v, uint32_t n) {
 // entries of frames before lo, are skipped) and then, if c_now is not
 // kCodeKeep, code c_now of frame t; writes pixel p's K indices to `idx`.
 //
-// With up to 8 slots and no flush among the codes, the frame that took slot j
-// last is kept as byte j of a 64-bit word: a code c puts its frame's number
-// (0..15, from t-15) at bit 8c, and kCodeKeep shifts out of both halves. That
+// With no flush among the codes, the frame that took slot j last is kept as
+// byte j of KM / 4 words: a code c puts its frame's number (0..15, from t-15)
+// at bit 8c, and kCodeKeep shifts out of every word. That
 // costs a fold about 10 instructions per code instead of 4 per code and slot:
 // VR K = 8 FP16 with the full bias 151 -> 138 us, HD K = 4 48.3 -> 46.9 us.
 template <int KM>
@@ -547,8 +545,9 @@ __device__ __forceinline__ void fold_store(const StreamDev& s, uint32_t* idx, in
   const int64_t pl = s.plane;
   uint32_t code[kRingFrames / 4];
 #pragma unroll
-  for (int w = 0; w < kRingFrames / 4; ++w) code[w] = in.code[w];
-  code[kRingFrames / 4 - 1] = (code[kRingFrames / 4 - 1] & 0x00ffffffu) | (static_cast<uint32_t>(c_now) << 24);
+  for (int w = 0; w < kRingFrames / 4; ++w)
+    code[w] = in.code[w];
+  code[kRingFrames / 4 - 1] |= static_cast<uint32_t>(c_now) << 24;
   // frames before lo keep (t - lo <= 15 frames are pending)
   const uint32_t skip = kRingFrames - 1 - (t - lo);
 #pragma unroll
@@ -564,17 +563,20 @@ __device__ __forceinline__ void fold_store(const StreamDev& s, uint32_t* idx, in
 #pragma unroll
   for (int j = 0; j < KM; ++j) v[j] = in.v[j];
   const uint32_t first = t - static_cast<uint32_t>(kRingFrames - 1);
-  if (KM <= 8 && flushed == 0u) {
-    uint32_t last0 = 0xffffffffu, last1 = 0xffffffffu;
+  if (flushed == 0u) {
+    uint32_t taken[(KM + 3) / 4];
+#pragma unroll
+    for (int w = 0; w < (KM + 3) / 4; ++w) taken[w] = 0xffffffffu;
 #pragma unroll
     for (int k = 0; k < kRingFrames; ++k) {
       const uint32_t at = 8u * ((code[k >> 2] >> (8 * (k & 3))) & 0xffu);
-      last0 = (last0 & ~shl_or_0(0xffu, at)) | shl_or_0(k, at);
-      if (KM > 4) last1 = (last1 & ~shl_or_0(0xffu, at - 32u)) | shl_or_0(k, at - 32u);
+#pragma unroll
+      for (int w = 0; w < (KM + 3) / 4; ++w)
+        taken[w] = (taken[w] & ~shl_or_0(0xffu, at - 32u * w)) | shl_or_0(k, at - 32u * w);
     }
 #pragma unroll
     for (int j = 0; j < KM; ++j) {
-      const uint32_t k = ((j < 4 ? last0 : last1) >> (8 * (j & 3))) & 0xffu;
+      const uint32_t k = (taken[j >> 2] >> (8 * (j & 3))) & 0xffu;
       if (k != 0xffu) v[j] = first + k;
     }
   } else {

@@ -57,7 +57,7 @@ uint32_t* wrs_status_word(const wrs_ctx* x);
 size_t wrs_pipe_smem_bytes(int K, bool f16, int px, int stages, bool resolve);
 bool wrs_pipe_supported(const wrs_ctx* x, const float* frame, int64_t pitch, const float* out);
 cudaError_t wrs_launch_pipe(const wrs::StreamDev& s, const wrs::FrameDev& f, bool f16, int px,
-                            int stages, int ctas_per_sm, uint32_t* status,
+                            int stages, int sms, int ctas_per_sm, uint32_t* status,
                             uint64_t timeout_ns, uint32_t extra_tx, cudaStream_t st);
 void wrs_default_pipe(int K, bool f16, int* px, int* stages);
 
@@ -83,7 +83,8 @@ int wrs_fov_check_source(const float* d_img, int64_t pitch, const void* d_mip, s
                    int32_t filter, wrs::FovDev* fv);
 // The pipelined kernel foveating the frame as it reads it (filter: WRS_FILTER_*).
 cudaError_t wrs_launch_pipe_fov(const wrs::StreamDev& s, const wrs::FrameDev& f,
-                                const wrs::FovDev& fv, int filter, bool f16, int stages, int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
+                                const wrs::FovDev& fv, int filter, bool f16, int stages, int sms,
+                                int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
                                 cudaStream_t st);
 cudaError_t wrs_launch_push(const wrs::StreamDev& s, const wrs::FrameDev& f, int block, int px,
                             bool f16, cudaStream_t st);

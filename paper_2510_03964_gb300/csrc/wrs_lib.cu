@@ -462,7 +462,7 @@ extern "C" int wrs_push_frame(wrs_ctx* x, const float* d_frame, int64_t pitch, f
       px = 1;  // a thread's pixels lie in one row: see wrs_pipe_supported
       stages = wrs_default_stages(x->cfg.K, x->cfg.color_fp16 != 0, 1);
     }
-    e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, px, stages, x->pipe_ctas,
+    e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, px, stages, x->sms, x->pipe_ctas,
                         wrs_status_word(x), x->timeout_ns, x->test_extra_tx,
                         static_cast<cudaStream_t>(stream));
   } else {
@@ -506,7 +506,7 @@ extern "C" int wrs_push_foveated(wrs_ctx* x, const float* d_img, int64_t img_pit
   int px = x->pipe_px, stages = x->pipe_stages;
   // the foveating form takes one pixel per thread: its own stage count then
   if (px != 1) stages = wrs_default_stages(x->cfg.K, x->cfg.color_fp16 != 0, 1);
-  cudaError_t e = wrs_launch_pipe_fov(s, f, fv, filter, x->cfg.color_fp16 != 0, stages, x->pipe_ctas,
+  cudaError_t e = wrs_launch_pipe_fov(s, f, fv, filter, x->cfg.color_fp16 != 0, stages, x->sms, x->pipe_ctas,
                                       wrs_status_word(x), x->timeout_ns,
                                       static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return wrs_cuda_fail(e, "wrs_push_foveated: launch");

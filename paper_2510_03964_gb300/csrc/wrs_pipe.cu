@@ -37,6 +37,7 @@ namespace {
 
 struct PipeArgs {
   int stages;
+  int queue;               // more tiles than CTAs that fit: see Ring::queue
   int resolve;             // copy weight/colour planes (fused resolve or full temporal bias)
   uint32_t* status;        // stream status word (WRS_OK or WRS_ERR_TIMEOUT)
   uint64_t timeout_ns;
@@ -44,23 +45,24 @@ struct PipeArgs {
 };
 
 constexpr int kConsumerWarps = 8;
-constexpr int kPipeThreads = (kConsumerWarps + 2) * 32;
+// FOVF >= 0: the frame is not copied but foveated from `fv` with filter FOVF
+// (WRS_FILTER_*) by two more warps; FOVF < 0: `fv` is unused.
+constexpr int producers(int fovf) { return fovf >= 0 ? 2 + wrs::kFovWarps : 2; }
+constexpr int pipe_threads(int fovf) { return (kConsumerWarps + producers(fovf)) * 32; }
 
 // Warp-specialised: warps 0..7 compute (consumers, PX pixels per thread), warp 8
 // issues copies and warp 9 draws uniforms. They meet only at the per-stage
 // full/empty barriers, never at a block-wide barrier.
-// FOVF >= 0: the frame is not copied but foveated by the consumers from `fv`
-// with filter FOVF (WRS_FILTER_*) as they compute; FOVF < 0: `fv` is unused.
 // Resident CTAs per SM the compiler is asked to fit: three for one or two
 // slots (their stages are small, and the extra warps hide the per-pixel
 // arithmetic's latency), two for one pixel per thread, else one.
-template <int KT, int PX>
+template <int KT, int PX, int FOVF>
 constexpr int pipe_min_blocks() {
-  return PX != 1 ? 1 : ((KT == 1 || KT == 2) ? 3 : 2);
+  return PX != 1 ? 1 : ((KT == 1 || KT == 2) && FOVF < 0 ? 3 : 2);
 }
 
 template <int KT, bool F16, int PX, bool LIT, int FOVF = -1>
-__global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
+__global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, FOVF>())
     pipe_kernel(const __grid_constant__ StreamDev s, const __grid_constant__ FrameDev f,
                 const PipeArgs a, const __grid_constant__ FovDev fv) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -69,13 +71,14 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
   const int K = KT > 0 ? KT : s.K;
   const bool resolve = a.resolve != 0;
   const StageLayout L = wrs::stage_layout(T, K, cs, resolve);
-  const wrs::Ring r = wrs::make_ring(smem, L.bytes, T, a.stages);
+  const wrs::Ring r = wrs::make_ring(smem, L.bytes, T, a.stages, a.queue != 0);
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
   __shared__ uint32_t failed;
+  if (warp == 0) wrs::init_ring(r, kConsumerWarps, producers(FOVF), lane);
+  wrs::grid_begin();
   if (tid == 0) {
-    wrs::init_ring(r, kConsumerWarps);
     // a wait of an earlier push gave up and the host has not yet seen it: the
     // reservoirs are undefined, so leave them (and the waits) alone
     failed = *reinterpret_cast<volatile const uint32_t*>(a.status);
@@ -97,6 +100,12 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
                         [&](uint32_t tile, uint8_t*, float* u, uint64_t* full, int ln) {
                           wrs::draw_tile_uniforms<T>(s, f, static_cast<int64_t>(tile) * T, u, full, ln);
                         });
+  } else if (FOVF >= 0 && warp >= kConsumerWarps + 2) {
+    if constexpr (FOVF >= 0)
+      wrs::produce<false>(r, a.timeout_ns, lane,
+                          [&](uint32_t tile, uint8_t* st, float*, uint64_t* full, int ln) {
+                            wrs::foveate_tile<FOVF>(s, f, fv, tile, st, full, warp - kConsumerWarps - 2, ln);
+                          });
   } else {
     constexpr int KM = wrs::FoldCap<KT>::value;
     const float d_f = wrs::fovea_density(s);
@@ -109,7 +118,7 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
           wrs::tile_ahead<KM, PX, (KT > 2)>(s, f, px);
         },
         [&](uint8_t* st, const float* u) {
-          replaced += wrs::compute_tile<KT, F16, PX, T, LIT, FOVF>(s, f, fv, st, u, px, d_f, tid);
+          replaced += wrs::compute_tile<KT, F16, PX, T, LIT>(s, f, st, u, px, d_f, tid);
         });
   }
   __syncthreads();
@@ -121,72 +130,83 @@ __global__ void __launch_bounds__(kPipeThreads, pipe_min_blocks<KT, PX>())
 }
 
 template <int KT, bool F16, int PX, bool LIT = false, int FOVF = -1>
-cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int ctas_per_sm,
+cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int sms, int ctas_per_sm,
                           cudaStream_t st, const FovDev& fv = FovDev{}) {
   constexpr int T = kConsumerWarps * 32 * PX;
   const StageLayout L = wrs::stage_layout(T, s.K, F16 ? 2 : 4, a.resolve != 0);
   size_t smem = wrs::ring_bytes(L.bytes, T, a.stages);
-  // per instantiation and device: the whole budget allowed once
-  static bool configured[64] = {};
+  // per instantiation and device: the whole budget allowed once, and how many
+  // CTAs of the last shared-memory size fit on the device
+  struct Fit {
+    size_t smem = 0;
+    int ctas = 0;
+  };
+  static Fit fits[64];
   static std::mutex lock;
+  const auto kernel = pipe_kernel<KT, F16, PX, LIT, FOVF>;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  int fit;
   {
     std::lock_guard<std::mutex> hold(lock);
-    if (!configured[dev]) {
-      e = cudaFuncSetAttribute(pipe_kernel<KT, F16, PX, LIT, FOVF>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBudget));
+    Fit& known = fits[dev];
+    if (known.smem == 0) {
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBudget));
       if (e != cudaSuccess) return e;
-      configured[dev] = true;
     }
+    if (known.smem != smem) {
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&known.ctas, kernel, pipe_threads(FOVF), smem);
+      if (e != cudaSuccess) return e;
+      known.smem = smem;
+    }
+    fit = known.ctas;
   }
-  int fit = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, pipe_kernel<KT, F16, PX, LIT, FOVF>,
-                                                    kPipeThreads, smem);
-  if (e != cudaSuccess) return e;
   if (fit < 1) return cudaErrorInvalidConfiguration;
   // fewer CTAs per SM than fit: a larger shared-memory request keeps the others out
-  if (ctas_per_sm > 0 && ctas_per_sm < fit) smem = wrs::smem_for_ctas(smem, ctas_per_sm);
+  if (ctas_per_sm > 0 && ctas_per_sm < fit) {
+    smem = wrs::smem_for_ctas(smem, ctas_per_sm);
+    fit = ctas_per_sm;
+  }
   const int64_t tiles = (static_cast<int64_t>(s.hw) + T - 1) / T;
-  pipe_kernel<KT, F16, PX, LIT, FOVF><<<static_cast<unsigned>(tiles), kPipeThreads, smem, st>>>(s, f, a, fv);
-  return cudaGetLastError();
+  a.queue = tiles > static_cast<int64_t>(fit) * sms ? 1 : 0;
+  return wrs_launch_early(kernel, dim3(static_cast<unsigned>(tiles)), pipe_threads(FOVF), smem, st, s, f, a, fv);
 }
 
 // The foveating form: one pixel per thread (the default tile), K = 4, 8 or
 // any other through the generic instantiation, and the literal rule.
 template <bool F16, int FILTER>
 cudaError_t launch_pipe_fov_k(const StreamDev& s, const FrameDev& f, const FovDev& fv,
-                              const PipeArgs& a, int ctas, cudaStream_t st) {
-  if (s.literal) return launch_pipe_t<1, F16, 1, true, FILTER>(s, f, a, ctas, st, fv);
+                              const PipeArgs& a, int sms, int ctas, cudaStream_t st) {
+  if (s.literal) return launch_pipe_t<1, F16, 1, true, FILTER>(s, f, a, sms, ctas, st, fv);
   switch (s.K) {
-    case 4: return launch_pipe_t<4, F16, 1, false, FILTER>(s, f, a, ctas, st, fv);
-    case 8: return launch_pipe_t<8, F16, 1, false, FILTER>(s, f, a, ctas, st, fv);
-    default: return launch_pipe_t<0, F16, 1, false, FILTER>(s, f, a, ctas, st, fv);
+    case 4: return launch_pipe_t<4, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
+    case 8: return launch_pipe_t<8, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
+    default: return launch_pipe_t<0, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
   }
 }
 
 template <int KT, bool F16, bool LIT = false>
-cudaError_t launch_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int ctas,
+cudaError_t launch_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
                             cudaStream_t st) {
   switch (px) {
-    case 4: return launch_pipe_t<KT, F16, 4, LIT>(s, f, a, ctas, st);
-    case 2: return launch_pipe_t<KT, F16, 2, LIT>(s, f, a, ctas, st);
-    default: return launch_pipe_t<KT, F16, 1, LIT>(s, f, a, ctas, st);
+    case 4: return launch_pipe_t<KT, F16, 4, LIT>(s, f, a, sms, ctas, st);
+    case 2: return launch_pipe_t<KT, F16, 2, LIT>(s, f, a, sms, ctas, st);
+    default: return launch_pipe_t<KT, F16, 1, LIT>(s, f, a, sms, ctas, st);
   }
 }
 
 template <bool F16>
-cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int ctas,
+cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
                            cudaStream_t st) {
-  if (s.literal) return launch_pipe_px<1, F16, true>(s, f, a, px, ctas, st);
+  if (s.literal) return launch_pipe_px<1, F16, true>(s, f, a, px, sms, ctas, st);
   switch (s.K) {
-    case 1: return launch_pipe_px<1, F16>(s, f, a, px, ctas, st);
-    case 2: return launch_pipe_px<2, F16>(s, f, a, px, ctas, st);
-    case 4: return launch_pipe_px<4, F16>(s, f, a, px, ctas, st);
-    case 8: return launch_pipe_px<8, F16>(s, f, a, px, ctas, st);
-    default: return launch_pipe_px<0, F16>(s, f, a, px, ctas, st);
+    case 1: return launch_pipe_px<1, F16>(s, f, a, px, sms, ctas, st);
+    case 2: return launch_pipe_px<2, F16>(s, f, a, px, sms, ctas, st);
+    case 4: return launch_pipe_px<4, F16>(s, f, a, px, sms, ctas, st);
+    case 8: return launch_pipe_px<8, F16>(s, f, a, px, sms, ctas, st);
+    default: return launch_pipe_px<0, F16>(s, f, a, px, sms, ctas, st);
   }
 }
 
@@ -209,7 +229,7 @@ bool wrs_pipe_supported(const wrs_ctx* x, const float* frame, int64_t pitch, con
 }
 
 cudaError_t wrs_launch_pipe_fov(const StreamDev& s, const FrameDev& f, const FovDev& fv, int filter,
-                                bool f16, int stages, int ctas_per_sm, uint32_t* status,
+                                bool f16, int stages, int sms, int ctas_per_sm, uint32_t* status,
                                 uint64_t timeout_ns, cudaStream_t st) {
   PipeArgs a;
   a.stages = stages;
@@ -218,14 +238,14 @@ cudaError_t wrs_launch_pipe_fov(const StreamDev& s, const FrameDev& f, const Fov
   a.timeout_ns = timeout_ns;
   a.extra_tx = 0;
   if (filter == WRS_FILTER_BOX)
-    return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BOX>(s, f, fv, a, ctas_per_sm, st)
-               : launch_pipe_fov_k<false, WRS_FILTER_BOX>(s, f, fv, a, ctas_per_sm, st);
-  return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BILINEAR>(s, f, fv, a, ctas_per_sm, st)
-             : launch_pipe_fov_k<false, WRS_FILTER_BILINEAR>(s, f, fv, a, ctas_per_sm, st);
+    return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, st)
+               : launch_pipe_fov_k<false, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, st);
+  return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, st)
+             : launch_pipe_fov_k<false, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, st);
 }
 
 cudaError_t wrs_launch_pipe(const StreamDev& s, const FrameDev& f, bool f16, int px, int stages,
-                            int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
+                            int sms, int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
                             uint32_t extra_tx, cudaStream_t st) {
   PipeArgs a;
   a.stages = stages;
@@ -233,6 +253,6 @@ cudaError_t wrs_launch_pipe(const StreamDev& s, const FrameDev& f, bool f16, int
   a.status = status;
   a.timeout_ns = timeout_ns;
   a.extra_tx = extra_tx;
-  return f16 ? launch_pipe_k<true>(s, f, a, px, ctas_per_sm, st)
-             : launch_pipe_k<false>(s, f, a, px, ctas_per_sm, st);
+  return f16 ? launch_pipe_k<true>(s, f, a, px, sms, ctas_per_sm, st)
+             : launch_pipe_k<false>(s, f, a, px, sms, ctas_per_sm, st);
 }

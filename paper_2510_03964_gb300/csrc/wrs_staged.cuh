@@ -54,17 +54,6 @@ __device__ __forceinline__ void fence_stage_writes() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// Whether pixels p .. p+PX-1 have their history flushed this frame (bit i).
-template <int PX>
-__device__ __forceinline__ uint32_t flush_bits(const FrameDev& f, uint32_t p) {
-  uint32_t bits = 0;
-  if (f.fov != nullptr) {
-#pragma unroll
-    for (int i = 0; i < PX; ++i) bits |= f.fov[static_cast<int64_t>(p) + i] == 0xFFu ? 1u << i : 0u;
-  }
-  return bits;
-}
-
 // Checked build: the entries a thread's PX pixels at p (tile entry tl) use.
 template <int PX, int T>
 __device__ __forceinline__ bool staged_in_bounds(const StreamDev& s, uint32_t p, int tl, int x, int y) {
