@@ -209,7 +209,9 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     e.code = code_of(x->cfg);
     tiles += (static_cast<int64_t>(e.s.hw) + T - 1) / T;
     const bool records = out != nullptr || x->cfg.temporal_bias == 2;
-    const uint32_t sb = wrs::stage_layout(T, x->cfg.K, x->cfg.color_fp16 ? 2 : 4, records).bytes;
+    const uint32_t sb = wrs::stage_layout(T, x->cfg.K, x->cfg.color_fp16 ? 2 : 4, records,
+                                          x->cfg.update_rule == WRS_RULE_LITERAL)
+                            .bytes;
     if (sb > stage_bytes) stage_bytes = sb;
   }
   if (tiles > 0x7FFFFFFF) return wrs_fail(WRS_ERR_ARG, "batch too large");

@@ -95,7 +95,7 @@ __device__ __forceinline__ void produce_tile(const BatchEntry& e, int64_t p0, ui
   const int K = KT > 0 ? KT : e.s.K;
   const int cs = CS > 0 ? CS : (entry_f16(e) ? 2 : 4);
   const bool resolve = stage_records(e);
-  const StageLayout L = wrs::stage_layout(T, K, cs, resolve);
+  const StageLayout L = wrs::stage_layout(T, K, cs, resolve, KT == 0 && e.s.literal != 0);
   wrs::issue_tile_copies<T>(e.s, e.f, K, cs, resolve, L, st, full, p0, 0u, ln, COPY_FRAME, stage_cap);
 }
 

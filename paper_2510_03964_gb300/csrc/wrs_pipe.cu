@@ -54,15 +54,19 @@ constexpr int pipe_threads(int fovf) { return (kConsumerWarps + producers(fovf))
 // issues copies and warp 9 draws uniforms. They meet only at the per-stage
 // full/empty barriers, never at a block-wide barrier.
 // Resident CTAs per SM the compiler is asked to fit: three for one or two
-// slots (their stages are small, and the extra warps hide the per-pixel
-// arithmetic's latency), two for one pixel per thread, else one.
-template <int KT, int PX, int FOVF>
+// slots and one pixel per thread and for the literal rule at up to two (their
+// stages are small, and the extra warps hide the per-pixel arithmetic's
+// latency: 4K literal rule, 24 against 16 consumer warps per SM, 68.7 -> 63.9 us), two for
+// one pixel per thread, else one.
+template <int KT, int PX, bool LIT, int FOVF>
 constexpr int pipe_min_blocks() {
-  return PX != 1 ? 1 : ((KT == 1 || KT == 2) && FOVF < 0 ? 3 : 2);
+  if (FOVF >= 0) return 2;
+  if (LIT ? PX <= 2 : (KT == 1 || KT == 2) && PX == 1) return 3;
+  return PX == 1 ? 2 : 1;
 }
 
 template <int KT, bool F16, int PX, bool LIT, int FOVF = -1>
-__global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, FOVF>())
+__global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, LIT, FOVF>())
     pipe_kernel(const __grid_constant__ StreamDev s, const __grid_constant__ FrameDev f,
                 const PipeArgs a, const __grid_constant__ FovDev fv) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -70,7 +74,7 @@ __global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, FO
   constexpr int cs = F16 ? 2 : 4;
   const int K = KT > 0 ? KT : s.K;
   const bool resolve = a.resolve != 0;
-  const StageLayout L = wrs::stage_layout(T, K, cs, resolve);
+  const StageLayout L = wrs::stage_layout(T, K, cs, resolve, LIT);
   const wrs::Ring r = wrs::make_ring(smem, L.bytes, T, a.stages, a.queue != 0);
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
@@ -133,7 +137,7 @@ template <int KT, bool F16, int PX, bool LIT = false, int FOVF = -1>
 cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int sms, int ctas_per_sm,
                           cudaStream_t st, const FovDev& fv = FovDev{}) {
   constexpr int T = kConsumerWarps * 32 * PX;
-  const StageLayout L = wrs::stage_layout(T, s.K, F16 ? 2 : 4, a.resolve != 0);
+  const StageLayout L = wrs::stage_layout(T, s.K, F16 ? 2 : 4, a.resolve != 0, LIT);
   size_t smem = wrs::ring_bytes(L.bytes, T, a.stages);
   // per instantiation and device: the whole budget allowed once, and how many
   // CTAs of the last shared-memory size fit on the device
@@ -212,10 +216,10 @@ cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs&
 
 }  // namespace
 
-// Shared memory one CTA of the pipelined kernel needs.
+// Shared memory one CTA of the pipelined kernel needs (the literal rule: less).
 size_t wrs_pipe_smem_bytes(int K, bool f16, int px, int stages, bool resolve) {
   const int T = kConsumerWarps * 32 * px;
-  return wrs::ring_bytes(wrs::stage_layout(T, K, f16 ? 2 : 4, resolve).bytes, T, stages);
+  return wrs::ring_bytes(wrs::stage_layout(T, K, f16 ? 2 : 4, resolve, false).bytes, T, stages);
 }
 
 // Frames the bulk copies can read: rows without padding, 16-byte aligned.

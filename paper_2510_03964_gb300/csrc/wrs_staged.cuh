@@ -27,23 +27,27 @@ namespace wrs {
 // Byte offsets of one stage's planes in shared memory (tile of T pixels).
 // cs = 2 (FP16 colour: K planes of the weights' low 16 bits, then K planes of
 // 8-byte records {r, g, b, w_hi}) or 4 (FP32 colour: K float4 {w, r, g, b}
-// record planes, starting at `col`; `wt` == `col`).
+// record planes, starting at `col`; `wt` == `col`). The literal rule has no P
+// and no key planes: its 512-pixel stages of 18 KB let three CTAs with four
+// stages share an SM.
 struct StageLayout {
   uint32_t frame, W, P, key, wt, col, bytes;
 };
 
-__host__ __device__ __forceinline__ StageLayout stage_layout(int T, int K, int cs, bool resolve) {
+__host__ __device__ __forceinline__ StageLayout stage_layout(int T, int K, int cs, bool resolve,
+                                                              bool literal) {
   StageLayout L;
   L.frame = 0;
   L.W = 12u * T;
   L.P = L.W + 4u * T;
-  L.key = L.P + 4u * T;
+  L.key = L.P + (literal ? 0u : 4u * T);
+  const uint32_t keys = literal ? 0u : 4u * K * T;
   if (cs == 2) {
-    L.wt = L.key + 4u * K * T;
+    L.wt = L.key + keys;
     L.col = L.wt + (resolve ? 2u * K * T : 0u);
     L.bytes = L.col + (resolve ? 8u * K * T : 0u);
   } else {
-    L.wt = L.col = L.key + 4u * K * T;
+    L.wt = L.col = L.key + keys;
     L.bytes = L.col + (resolve ? 16u * K * T : 0u);
   }
   return L;
@@ -83,7 +87,7 @@ __device__ __forceinline__ int push_staged(const StreamDev& s, const FrameDev& f
   const int64_t pl = s.plane;
   const int tl = tid * PX;
   if (!staged_in_bounds<PX, T>(s, p, tl, x, y)) return 0;
-  const StageLayout L = stage_layout(T, K, F16 ? 2 : 4, true);
+  const StageLayout L = stage_layout(T, K, F16 ? 2 : 4, true, false);
   float* key = reinterpret_cast<float*>(st + L.key) + tl;
   uint16_t* wt = reinterpret_cast<uint16_t*>(st + L.wt);
   uint8_t* col = st + L.col;
@@ -224,7 +228,7 @@ __device__ __forceinline__ int push_staged_literal(const StreamDev& s, const Fra
                                                    uint32_t flush) {
   const int tl = tid * PX;
   if (!staged_in_bounds<PX, T>(s, p, tl, x, y)) return 0;
-  const StageLayout L = stage_layout(T, 1, F16 ? 2 : 4, true);
+  const StageLayout L = stage_layout(T, 1, F16 ? 2 : 4, true, true);
   const bool records = f.out != nullptr || s.bias == 2;
   float rgb[PX][3], Wv[PX], a[PX], r[PX], g[PX], b[PX], o[PX][3];
   load_rgb<PX>(reinterpret_cast<const float*>(st + L.frame) + 3 * tl, rgb);
