@@ -45,6 +45,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+// `bytes` (multiple of 16, 16-byte aligned) of global memory into the L2
+__device__ __forceinline__ void bulk_prefetch(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -78,7 +83,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 
 // Warp-wide: lane 0 arms `bar` for the tile's bytes (plus extra_tx, which is
 // non-zero only to test the timeout path), then the lanes issue one bulk copy
-// per plane segment. The tile starts at pixel p0 (a multiple of T >= 256);
+// per plane segment, and bring what the tile's fold will read into the L2. The tile starts at pixel p0 (a multiple of T >= 256);
 // requires frame rows without padding and 16-byte aligned frame and state
 // planes. A bulk copy moves whole 16 bytes, four pixels of the frame: up to
 // three last pixels of an image come by plain loads. copy_frame = false leaves the frame segment to the
@@ -153,13 +158,36 @@ __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const Fram
                8u * n, bar);
     }
   }
+  if constexpr (T == 256) {
+    if (K > 2 && folds_now(f, p0)) {
+      // the code rows of the last 15 frames and the K index rows: the consumers
+      // load them when they come to the tile, S tiles later (HD K = 4 43.9 ->
+      // 42.6 us)
+      const int c = lane < kRingFrames - 1 ? lane : lane - (kRingFrames - 1);
+      if (lane < kRingFrames - 1)
+        bulk_prefetch(s.maps + static_cast<int64_t>((f.t - 1u - c) & kRingMask) * pl + p0, n);
+      else if (c < K)
+        bulk_prefetch(s.idx + c * pl + p0, 4u * n);
+    }
+  }
 }
 
 // The tile's uniforms, drawn by one warp: one Philox block per 4 pixels,
-// written to u[0 .. T-1], then the warp's arrival on `bar`.
+// written to u[0 .. T-1]; with a flush map its entries of the tile go to the T
+// bytes behind them. Then the warp's arrival on `bar`. The consumers loaded
+// their own flush-map bytes before: a wait on DRAM in every tile that the wait
+// for the stage seldom covered, 1365 x 767 K = 4 with flushes 29.7 -> 27.5 us.
 template <int T>
-__device__ __forceinline__ void draw_tile_uniforms(const StreamDev& s, const FrameDev& f,
-                                                   int64_t p0, float* u, uint64_t* bar, int lane) {
+__device__ __forceinline__ void draw_tile(const StreamDev& s, const FrameDev& f, int64_t p0, float* u,
+                                          uint64_t* bar, int lane) {
+  uint8_t fov[T / 32];
+  if (f.fov != nullptr) {
+#pragma unroll
+    for (int i = 0; i < T / 32; ++i) {
+      const int64_t p = p0 + 32 * i + lane;
+      fov[i] = p < s.hw ? f.fov[p] : 0u;
+    }
+  }
 #pragma unroll
   for (int q = lane; q < T / 4; q += 32) {
     const uint32_t blk = static_cast<uint32_t>((p0 >> 2) + q);
@@ -171,19 +199,22 @@ __device__ __forceinline__ void draw_tile_uniforms(const StreamDev& s, const Fra
     v.w = unit_uniform(b.w);
     reinterpret_cast<float4*>(u)[q] = v;
   }
+  if (f.fov != nullptr) {
+    uint8_t* flags = reinterpret_cast<uint8_t*>(u + T);
+#pragma unroll
+    for (int i = 0; i < T / 32; ++i) flags[32 * i + lane] = fov[i];
+  }
   __syncwarp();
   if (lane == 0) mbar_arrive(bar);
 }
 
 // What a consumer thread of a tile knows before the tile has landed: its first
-// pixel p = (x, y) (no pixel if p >= hw), the flush-map entries of its PX
-// pixels and, in the band this frame folds, the fold's inputs. Loaded ahead of
-// the wait and first used after it, so that their latency passes while the
-// tile is still in flight.
+// pixel p = (x, y) (no pixel if p >= hw) and, in the band this frame folds, the
+// fold's inputs, loaded ahead of the wait, so that their latency passes while
+// the tile is still in flight.
 template <int KM>
 struct TilePx {
   uint32_t p;
-  uint32_t fov[4];  // the pixels' flush-map entries
   int x, y;
   bool folding;
   FoldIn<KM> fold;
@@ -192,14 +223,8 @@ struct TilePx {
 // Fills t for the pixels at t.p (t.x and t.y already set).
 template <int KM, int PX, bool FOLD>
 __device__ __forceinline__ void tile_ahead(const StreamDev& s, const FrameDev& f, TilePx<KM>& t) {
-#pragma unroll
-  for (int i = 0; i < PX; ++i) t.fov[i] = 0u;
   t.folding = false;
   if (t.p >= static_cast<uint32_t>(s.hw)) return;
-  if (f.fov != nullptr) {
-#pragma unroll
-    for (int i = 0; i < PX; ++i) t.fov[i] = f.fov[static_cast<int64_t>(t.p) + i];
-  }
   if constexpr (FOLD && PX == 1) {
     if (s.K > 2 && s.K <= KM && folds_now(f, t.p)) {
       fold_load(s, s.idx, s.K, f.t, t.p, t.fold);
@@ -216,8 +241,11 @@ __device__ __forceinline__ int compute_tile(const StreamDev& s, const FrameDev& 
                                             const float* u, const TilePx<KM>& t, float d_f, int tid) {
   if (t.p >= static_cast<uint32_t>(s.hw)) return 0;
   uint32_t flush = 0;
+  if (f.fov != nullptr) {
+    const uint8_t* flags = reinterpret_cast<const uint8_t*>(u + T) + tid * PX;
 #pragma unroll
-  for (int i = 0; i < PX; ++i) flush |= t.fov[i] == 0xFFu ? 1u << i : 0u;
+    for (int i = 0; i < PX; ++i) flush |= flags[i] == 0xFFu ? 1u << i : 0u;
+  }
   if constexpr (LIT)
     return push_staged_literal<F16, PX, T>(s, f, st, u, t.p, t.x, t.y, d_f, tid, flush);
   else
@@ -305,12 +333,12 @@ constexpr int kMaxStages = 8;
 constexpr int kAnswers = kMaxStages + 2;
 
 // Shared-memory ring of S stages, each holding one tile's planes followed by
-// its uniforms, then the S "full" and S "empty" barriers, and the answers of
+// its uniforms and, if some frame has a flush map, its flush-map entries, then the S "full" and S "empty" barriers, and the answers of
 // the work queue with theirs.
 struct Ring {
   uint8_t* base;
   uint32_t stage_bytes;  // planes of the largest tile layout used
-  uint32_t stride;       // stage_bytes + 4 * T
+  uint32_t stride;       // stage_bytes + 4 * T (+ T with flush maps)
   int S;
   bool queue;            // the grid has more tiles than CTAs that fit: ask for more
   uint64_t* full;
@@ -323,17 +351,31 @@ struct Ring {
   __device__ float* u(int i) const { return reinterpret_cast<float*>(base + i * stride + stage_bytes); }
 };
 
-__host__ __device__ __forceinline__ size_t ring_bytes(uint32_t stage_bytes, int T, int S) {
-  return static_cast<size_t>(S) * (stage_bytes + 4u * T) + 16u * S + 24u * kAnswers + 16u;
+__host__ __device__ __forceinline__ size_t ring_bytes(uint32_t stage_bytes, int T, int S, bool maps) {
+  return static_cast<size_t>(S) * (stage_bytes + (maps ? 5u : 4u) * T) + 16u * S + 24u * kAnswers + 16u;
+}
+
+// Stages that keep as many CTAs of a ring with flush maps on an SM as fit
+// without them (one CTA at least).
+__host__ inline int stages_with_maps(uint32_t stage_bytes, int T, int S) {
+  constexpr size_t kSmPerSm = 228 * 1024, kReservedPerCta = 2048, kMost = 226 * 1024;
+  const size_t plain = ring_bytes(stage_bytes, T, S, false);
+  const size_t ctas = kSmPerSm / (plain + kReservedPerCta);
+  while (S > 1) {
+    const size_t smem = ring_bytes(stage_bytes, T, S, true);
+    if (smem <= kMost && kSmPerSm / (smem + kReservedPerCta) >= ctas) break;
+    --S;
+  }
+  return S;
 }
 
 __device__ __forceinline__ Ring make_ring(uint8_t* smem, uint32_t stage_bytes, int T, int S,
-                                          bool queue) {
+                                          bool queue, bool maps) {
   Ring r;
   r.queue = queue;
   r.base = smem;
   r.stage_bytes = stage_bytes;
-  r.stride = stage_bytes + 4u * T;
+  r.stride = stage_bytes + (maps ? 5u : 4u) * T;
   r.S = S;
   r.answer = reinterpret_cast<uint4*>(smem + static_cast<size_t>(S) * r.stride);
   r.full = reinterpret_cast<uint64_t*>(r.answer + kAnswers);

@@ -158,6 +158,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   const int px = fov ? 1 : b->px;
   const int T = 256 * px;
   int64_t tiles = 0;
+  bool maps = false;
   uint32_t stage_bytes = 0;
   int device = -1;
   for (int i = 0; i < n; ++i) {
@@ -200,6 +201,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     e.f.pitch = 3 * static_cast<int64_t>(x->cfg.width);
     e.f.fov = d_fov_maps ? d_fov_maps[i] : nullptr;
     e.f.out = out;
+    maps = maps || e.f.fov != nullptr;
     e.f.gx = gx;
     e.f.gy = gy;
     e.f.t = x->t;
@@ -220,15 +222,20 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     // as many stages (up to 4) as keep two CTAs on an SM, else what one CTA holds
     constexpr size_t kSmPerSm = 228 * 1024, kReservedPerCta = 1024;
     stages = 4;
-    while (stages > 2 && 2 * (wrs::ring_bytes(stage_bytes, T, stages) + kReservedPerCta) > kSmPerSm)
+    while (stages > 2 && 2 * (wrs::ring_bytes(stage_bytes, T, stages, false) + kReservedPerCta) > kSmPerSm)
       --stages;
-    while (stages > 1 && wrs::ring_bytes(stage_bytes, T, stages) > kSmemBudget) --stages;
+    while (stages > 1 && wrs::ring_bytes(stage_bytes, T, stages, false) > kSmemBudget) --stages;
   }
-  size_t smem = wrs::ring_bytes(stage_bytes, T, stages);
+  size_t smem = wrs::ring_bytes(stage_bytes, T, stages, false);
   if (smem > kSmemBudget)
     return wrs_fail(WRS_ERR_ARG, "%d stages of %u B exceed shared memory", stages, stage_bytes);
+  if (maps) {
+    stages = wrs::stages_with_maps(stage_bytes, T, stages);
+    smem = wrs::ring_bytes(stage_bytes, T, stages, true);
+  }
   a.n = n;
   a.stages = stages;
+  a.maps = maps ? 1 : 0;
   a.stage_bytes = stage_bytes;
   a.timeout_ns = ctxs[0]->timeout_ns;
 

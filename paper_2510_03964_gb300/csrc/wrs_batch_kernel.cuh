@@ -38,6 +38,7 @@ __device__ __forceinline__ bool stage_records(const BatchEntry& e) {
 struct BatchArgs {
   int n;
   int queue;             // more tiles than CTAs that fit: see Ring::queue
+  int maps;              // some frame has a flush map: see Ring
   int stages;
   uint32_t stage_bytes;  // largest stage of any stream in the batch
   uint64_t timeout_ns;
@@ -112,7 +113,7 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
   __shared__ float d_f_s[kMaxBatch];                    // per stream: density at the fovea edge
   __shared__ uint32_t failed_s[kMaxBatch];              // per stream: an earlier wait gave up
   constexpr int T = kConsumerWarps * 32 * PX;
-  const wrs::Ring r = wrs::make_ring(smem, a.stage_bytes, T, a.stages, a.queue != 0);
+  const wrs::Ring r = wrs::make_ring(smem, a.stage_bytes, T, a.stages, a.queue != 0, a.maps != 0);
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
                         [&](uint32_t g, uint8_t*, float* u, uint64_t* full, int ln) {
       pe = entry_after(a, g, pe);
       const BatchEntry& e = a.e[pe];
-      wrs::draw_tile_uniforms<T>(e.s, e.f, static_cast<int64_t>(g - e.tile0) * T, u, full, ln);
+      wrs::draw_tile<T>(e.s, e.f, static_cast<int64_t>(g - e.tile0) * T, u, full, ln);
     });
   } else if (FOVF >= 0 && warp >= kConsumerWarps + 2) {
     int pe = 0;

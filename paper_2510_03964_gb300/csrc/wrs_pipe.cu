@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, LI
   const int K = KT > 0 ? KT : s.K;
   const bool resolve = a.resolve != 0;
   const StageLayout L = wrs::stage_layout(T, K, cs, resolve, LIT);
-  const wrs::Ring r = wrs::make_ring(smem, L.bytes, T, a.stages, a.queue != 0);
+  const wrs::Ring r = wrs::make_ring(smem, L.bytes, T, a.stages, a.queue != 0, f.fov != nullptr);
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, LI
   } else if (warp == kConsumerWarps + 1) {
     wrs::produce<false>(r, a.timeout_ns, lane,
                         [&](uint32_t tile, uint8_t*, float* u, uint64_t* full, int ln) {
-                          wrs::draw_tile_uniforms<T>(s, f, static_cast<int64_t>(tile) * T, u, full, ln);
+                          wrs::draw_tile<T>(s, f, static_cast<int64_t>(tile) * T, u, full, ln);
                         });
   } else if (FOVF >= 0 && warp >= kConsumerWarps + 2) {
     if constexpr (FOVF >= 0)
@@ -138,7 +138,8 @@ cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int
                           cudaStream_t st, const FovDev& fv = FovDev{}) {
   constexpr int T = kConsumerWarps * 32 * PX;
   const StageLayout L = wrs::stage_layout(T, s.K, F16 ? 2 : 4, a.resolve != 0, LIT);
-  size_t smem = wrs::ring_bytes(L.bytes, T, a.stages);
+  if (f.fov != nullptr) a.stages = wrs::stages_with_maps(L.bytes, T, a.stages);
+  size_t smem = wrs::ring_bytes(L.bytes, T, a.stages, f.fov != nullptr);
   // per instantiation and device: the whole budget allowed once, and how many
   // CTAs of the last shared-memory size fit on the device
   struct Fit {
@@ -219,7 +220,7 @@ cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs&
 // Shared memory one CTA of the pipelined kernel needs (the literal rule: less).
 size_t wrs_pipe_smem_bytes(int K, bool f16, int px, int stages, bool resolve) {
   const int T = kConsumerWarps * 32 * px;
-  return wrs::ring_bytes(wrs::stage_layout(T, K, f16 ? 2 : 4, resolve, false).bytes, T, stages);
+  return wrs::ring_bytes(wrs::stage_layout(T, K, f16 ? 2 : 4, resolve, false).bytes, T, stages, false);
 }
 
 // Frames the bulk copies can read: rows without padding, 16-byte aligned.
