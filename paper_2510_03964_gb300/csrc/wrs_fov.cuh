@@ -31,7 +31,7 @@ struct FovDev {
   const float* img;                     // [H][pitch] RGB triples
   int64_t pitch;
   int32_t nradii;                       // 1..WRS_MAX_MIP_LEVELS-1
-  float r2[WRS_MAX_MIP_LEVELS - 1];     // r_i * r_i, rounded once
+  float r2[WRS_MAX_MIP_LEVELS - 1];     // r_i * r_i, rounded once; infinite past nradii
   MipLevelDev lev[WRS_MAX_MIP_LEVELS];  // [1..nradii]; [0] unused (the image)
 };
 
@@ -59,8 +59,7 @@ __device__ __forceinline__ int ring_level(const FovDev& a, float gx, float dy2, 
   const float d2 = __fadd_rn(__fmul_rn(dx, dx), dy2);
   int L = 0;
 #pragma unroll
-  for (int i = 0; i < WRS_MAX_MIP_LEVELS - 1; ++i)
-    if (i < a.nradii) L += d2 > a.r2[i];
+  for (int i = 0; i < WRS_MAX_MIP_LEVELS - 1; ++i) L += d2 > a.r2[i] ? 1 : 0;
   return L;
 }
 
