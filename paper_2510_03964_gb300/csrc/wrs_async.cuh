@@ -83,12 +83,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 
 // Warp-wide: lane 0 arms `bar` for the tile's bytes (plus extra_tx, which is
 // non-zero only to test the timeout path), then the lanes issue one bulk copy
-// per plane segment, and bring what the tile's fold will read into the L2. The tile starts at pixel p0 (a multiple of T >= 256);
+// per plane segment. The tile starts at pixel p0 (a multiple of T >= 256);
 // requires frame rows without padding and 16-byte aligned frame and state
 // planes. A bulk copy moves whole 16 bytes, four pixels of the frame: up to
 // three last pixels of an image come by plain loads. copy_frame = false leaves the frame segment to the
 // consumers (they foveate the frame into it themselves).
-template <int T>
+// AHEAD: also bring what the tile's fold will read into the L2.
+template <int T, bool AHEAD>
 __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const FrameDev& f, int K,
                                                   int cs, bool resolve, const StageLayout& L,
                                                   uint8_t* stage, uint64_t* bar, int64_t p0,
@@ -158,7 +159,7 @@ __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const Fram
                8u * n, bar);
     }
   }
-  if constexpr (T == 256) {
+  if constexpr (T == 256 && AHEAD) {
     if (K > 2 && folds_now(f, p0)) {
       // the code rows of the last 15 frames and the K index rows: the consumers
       // load them when they come to the tile, S tiles later (HD K = 4 43.9 ->
@@ -168,6 +169,34 @@ __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const Fram
         bulk_prefetch(s.maps + static_cast<int64_t>((f.t - 1u - c) & kRingMask) * pl + p0, n);
       else if (c < K)
         bulk_prefetch(s.idx + c * pl + p0, 4u * n);
+    }
+  }
+}
+
+// The planes of the CTA's first tile into the L2 (the copies proper wait for
+// the stream's status word, a read of about 0.7 us: HD K = 4 42.8 -> 42.2 us).
+template <int T>
+__device__ __forceinline__ void prefetch_tile(const StreamDev& s, const FrameDev& f, int K, int cs,
+                                              bool resolve, int64_t p0, int lane) {
+  const int64_t pl = s.plane;
+  const int64_t rem = pl - p0;
+  if (p0 >= s.hw) return;
+  const uint32_t n = static_cast<uint32_t>(rem < T ? rem : T);
+  const int64_t rem_px = s.hw - p0;
+  const uint32_t np4 = static_cast<uint32_t>(rem_px < T ? rem_px : T) & ~3u;
+  if (lane == 0) {
+    if (f.frame != nullptr && np4 != 0u) bulk_prefetch(f.frame + 3 * p0, 12u * np4);
+    bulk_prefetch(s.W + p0, 4u * n);
+    if (!s.literal) bulk_prefetch(s.P + p0, 4u * n);
+  }
+  for (int j = lane; j < K; j += 32) {
+    if (!s.literal) bulk_prefetch(s.key + j * pl + p0, 4u * n);
+    if (!resolve) continue;
+    if (cs == 2) {
+      bulk_prefetch(s.wt + j * pl + p0, 2u * n);
+      bulk_prefetch(static_cast<const uint2*>(s.col) + j * pl + p0, 8u * n);
+    } else {
+      bulk_prefetch(static_cast<const float4*>(s.col) + j * pl + p0, 16u * n);
     }
   }
 }

@@ -97,7 +97,7 @@ __device__ __forceinline__ void produce_tile(const BatchEntry& e, int64_t p0, ui
   const int cs = CS > 0 ? CS : (entry_f16(e) ? 2 : 4);
   const bool resolve = stage_records(e);
   const StageLayout L = wrs::stage_layout(T, K, cs, resolve, KT == 0 && e.s.literal != 0);
-  wrs::issue_tile_copies<T>(e.s, e.f, K, cs, resolve, L, st, full, p0, 0u, ln, COPY_FRAME, stage_cap);
+  wrs::issue_tile_copies<T, false>(e.s, e.f, K, cs, resolve, L, st, full, p0, 0u, ln, COPY_FRAME, stage_cap);
 }
 
 // Warp-specialised like the single-stream pipelined kernel: warp 8 issues each
