@@ -447,10 +447,15 @@ __device__ __forceinline__ void store_rgb(float* dst, const float (&o)[N][3]) {
 // idx[j] and the state has no code ring: such kernels are bound by
 // instruction issue, not by DRAM, and at their low replacement rates the
 // ring's per-pixel work costs more than the scattered index writes it saves.
+//
+// A kernel's KT: its slot count, 0 for any number, or kUpTo8 for any number up
+// to 8 (loops over the slots are then unrolled as for 8 slots, each with a
+// uniform test, and the fold's inputs fit in the registers held over a wait).
+constexpr int kUpTo8 = -8;
 template <int KT>
 __device__ __forceinline__ bool direct_index(const StreamDev& s) {
   if constexpr (KT == 1 || KT == 2) return true;
-  else if constexpr (KT == 0) return s.K <= 2;
+  else if constexpr (KT <= 0) return s.K <= 2;
   else return false;
 }
 
@@ -498,7 +503,7 @@ struct FoldIn {
 // K): exactly KT, so that a kernel for few slots holds no unused registers.
 template <int KT>
 struct FoldCap {
-  static constexpr int value = (KT > 0 && KT <= 8) ? KT : WRS_MAX_K;
+  static constexpr int value = KT == kUpTo8 ? 8 : (KT > 0 && KT <= 8) ? KT : WRS_MAX_K;
 };
 
 template <int KT>

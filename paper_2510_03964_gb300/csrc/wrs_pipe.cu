@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, LI
         [&](uint32_t tile) {
           px.p = tile * T + tid * PX;
           wrs::row_col(s, static_cast<int>(px.p), px.y, px.x);
-          wrs::tile_ahead<KM, PX, (KT > 2)>(s, f, px);
+          wrs::tile_ahead<KM, PX, (KT > 2 || KT == wrs::kUpTo8)>(s, f, px);
         },
         [&](uint8_t* st, const float* u) {
           replaced += wrs::compute_tile<KT, F16, PX, T, LIT>(s, f, st, u, px, d_f, tid);
@@ -192,7 +192,9 @@ cudaError_t launch_pipe_fov_k(const StreamDev& s, const FrameDev& f, const FovDe
   switch (s.K) {
     case 4: return launch_pipe_t<4, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
     case 8: return launch_pipe_t<8, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
-    default: return launch_pipe_t<0, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
+    default:
+      if (s.K <= 8) return launch_pipe_t<wrs::kUpTo8, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
+      return launch_pipe_t<0, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
   }
 }
 
@@ -215,7 +217,11 @@ cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs&
     case 2: return launch_pipe_px<2, F16>(s, f, a, px, sms, ctas, st);
     case 4: return launch_pipe_px<4, F16>(s, f, a, px, sms, ctas, st);
     case 8: return launch_pipe_px<8, F16>(s, f, a, px, sms, ctas, st);
-    default: return launch_pipe_px<0, F16>(s, f, a, px, sms, ctas, st);
+    default:
+      // other slot counts: up to 8 unrolled with a test per slot, 9 to 16
+      // through run-time loops (184 x 143, K = 6: 4.8 us against 10.6)
+      if (px == 1 && s.K <= 8) return launch_pipe_t<wrs::kUpTo8, F16, 1>(s, f, a, sms, ctas, st);
+      return launch_pipe_px<0, F16>(s, f, a, px, sms, ctas, st);
   }
 }
 

@@ -84,6 +84,7 @@ __device__ __forceinline__ int push_staged(const StreamDev& s, const FrameDev& f
                                            int tid, uint32_t flush, const FoldIn<KM>* pre) {
   static_assert(4 % PX == 0, "pixels per thread must divide 4");
   const int K = KT > 0 ? KT : s.K;
+  const int n = KT == kUpTo8 ? 8 : K;  // bound of the unrolled loops
   const int64_t pl = s.plane;
   const int tl = tid * PX;
   if (!staged_in_bounds<PX, T>(s, p, tl, x, y)) return 0;
@@ -106,7 +107,8 @@ __device__ __forceinline__ int push_staged(const StreamDev& s, const FrameDev& f
 #pragma unroll
     for (int i = 0; i < PX; ++i) { n0[i] = n1[i] = n2[i] = dn[i] = 0.0f; }
 #pragma unroll 4
-    for (int j = 0; j < K; ++j) {
+    for (int j = 0; j < n; ++j) {
+      if (KT == kUpTo8 && j >= K) break;
       float a[PX], r[PX], g[PX], b[PX];
       load_slot<F16, PX>(wt, col, K, j, T, tl, a, r, g, b);
 #pragma unroll
@@ -164,7 +166,8 @@ __device__ __forceinline__ int push_staged(const StreamDev& s, const FrameDev& f
 #pragma unroll
   for (int i = 0; i < PX; ++i) kmax[i] = -1.0f;
 #pragma unroll 8
-  for (int j = 0; j < K; ++j) {
+  for (int j = 0; j < n; ++j) {
+    if (KT == kUpTo8 && j >= K) break;
     float kv[PX];
     load_f<PX>(key + j * T, kv);
 #pragma unroll
@@ -179,8 +182,8 @@ __device__ __forceinline__ int push_staged(const StreamDev& s, const FrameDev& f
     if (ks[i] < kmax[i]) {
       int jm = 0;
 #pragma unroll 8
-      for (int j = K - 1; j >= 0; --j)
-        if (key[j * T + i] == kmax[i]) jm = j;
+      for (int j = n - 1; j >= 0; --j)
+        if ((KT != kUpTo8 || j < K) && key[j * T + i] == kmax[i]) jm = j;
       replaced += 1;
       code = jm | dropped;
       s.key[jm * pl + q] = ks[i];
@@ -197,7 +200,8 @@ __device__ __forceinline__ int push_staged(const StreamDev& s, const FrameDev& f
 #pragma unroll
     for (int i = 0; i < PX; ++i) num[i][0] = num[i][1] = num[i][2] = den[i] = 0.0f;
 #pragma unroll 8
-    for (int j = 0; j < K; ++j) {
+    for (int j = 0; j < n; ++j) {
+      if (KT == kUpTo8 && j >= K) break;
       float a[PX], r[PX], g[PX], b[PX];
       load_slot<F16, PX>(wt, col, K, j, T, tl, a, r, g, b);
 #pragma unroll
