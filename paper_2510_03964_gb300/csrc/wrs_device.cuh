@@ -279,7 +279,14 @@ __device__ __forceinline__ void store_f(float* p, const float (&v)[N]) {
 // fourth half word (rec_hi = the record's second 32-bit word) and the low half
 // from the weight plane.
 __device__ __forceinline__ float slot_weight_f16(uint32_t rec_hi, uint32_t lo) {
-  return __uint_as_float((rec_hi & 0xffff0000u) | (lo & 0xffffu));
+  return __uint_as_float(__byte_perm(rec_hi, lo, 0x3254));
+}
+// The colour of an FP16 record {r, g, b, w_hi}.
+__device__ __forceinline__ void slot_colour_f16(uint2 rec, float& r, float& g, float& b) {
+  const float2 rg = __half22float2(*reinterpret_cast<const __half2*>(&rec.x));
+  r = rg.x;
+  g = rg.y;
+  b = __low2float(*reinterpret_cast<const __half2*>(&rec.y));
 }
 
 // Weight and colour of slot j for a group of N pixels whose first entry is at
@@ -298,9 +305,7 @@ __device__ __forceinline__ void load_slot(const uint16_t* wt, const void* col, i
     for (int i = 0; i < N; ++i) {
       const uint2 v = rec[i];
       a[i] = slot_weight_f16(v.y, lo[i]);
-      r[i] = __half2float(__ushort_as_half(static_cast<unsigned short>(v.x & 0xffffu)));
-      g[i] = __half2float(__ushort_as_half(static_cast<unsigned short>(v.x >> 16)));
-      b[i] = __half2float(__ushort_as_half(static_cast<unsigned short>(v.y & 0xffffu)));
+      slot_colour_f16(v, r[i], g[i], b[i]);
     }
   } else {
     const float4* rec = static_cast<const float4*>(col) + j * stride + at;
