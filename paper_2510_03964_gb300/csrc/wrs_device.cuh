@@ -32,7 +32,11 @@ constexpr float kFltMax = 3.40282346638528859812e+38f;
 constexpr float kLn2Hi = 0x1.62ep-1f;
 constexpr float kLn2Lo = 0x1.0bfbe8p-15f;
 constexpr float kLog2e = 0x1.715476p+0f;   // float nearest 1/ln 2
-constexpr float kSqrt2 = 0x1.6a09e6p+0f;   // float nearest sqrt 2
+constexpr uint32_t kSqrtHalfBits = 0x3f3504f4u;  // first float above half the float nearest sqrt 2
+// 1.5 * 2^23: adding it to |x| < 2^22 rounds x to an integer (nearest even) that
+// stands in the sum's low bits; no conversion instruction, whose latency (and
+// that of the rounding instruction) stands in every pixel's chain
+constexpr float kRound = 12582912.0f;
 // floats nearest 1/k! (k = 3..7) and 1/(2k+1) (k = 1..4)
 constexpr float kF3 = 0x1.555556p-3f, kF4 = 0x1.555556p-5f, kF5 = 0x1.111112p-7f,
                 kF6 = 0x1.6c16c2p-10f, kF7 = 0x1.a01a02p-13f;
@@ -57,7 +61,8 @@ __device__ __forceinline__ float ffma(float a, float b, float c) { return __fmaf
 // degree 7 in Horner form; times 2^n through the exponent field.
 __device__ __forceinline__ float exp_nonpos(float x) {
   x = fminf(fmaxf(x, -87.0f), 0.0f);
-  const float n = rintf(fmul(x, kLog2e));
+  const float t = fadd(fmul(x, kLog2e), kRound);  // n in the low bits
+  const float n = fsub(t, kRound);
   float r = ffma(-n, kLn2Hi, x);
   r = ffma(-n, kLn2Lo, r);
   float p = ffma(r, kF7, kF6);
@@ -67,20 +72,18 @@ __device__ __forceinline__ float exp_nonpos(float x) {
   p = ffma(r, p, 0.5f);
   p = ffma(r, p, 1.0f);
   p = ffma(r, p, 1.0f);
-  const int ni = __float2int_rn(n);
-  return fmul(p, __uint_as_float(static_cast<uint32_t>(ni + 127) << 23));
+  return fmul(p, __uint_as_float((__float_as_uint(t) + 127u) << 23));
 }
 
 // ln(u) for normal u > 0: u = m 2^e, m in [sqrt(1/2), sqrt 2); ln m = 2 atanh(s),
 // s = (m-1)/(m+1), series in s^2 to s^8/9.
 __device__ __forceinline__ float log_pos(float u) {
-  const uint32_t b = __float_as_uint(u);
-  int e = static_cast<int>((b >> 23) & 0xffu) - 127;
-  float m = __uint_as_float((b & 0x007fffffu) | 0x3f800000u);
-  if (m > kSqrt2) {
-    m = fmul(m, 0.5f);
-    e += 1;
-  }
+  // adding (1 - sqrt 1/2 in bits) carries into the exponent where the mantissa
+  // is above sqrt 2's; the exponent becomes a float by the integer in the low
+  // bits of 1.5 * 2^23
+  const uint32_t b = __float_as_uint(u) + (0x3f800000u - kSqrtHalfBits);
+  const float m = __uint_as_float((b & 0x007fffffu) + kSqrtHalfBits);
+  const float fe = fsub(__uint_as_float(__float_as_uint(kRound) + (b >> 23)), kRound + 127.0f);
   const float s = fdiv(fsub(m, 1.0f), fadd(m, 1.0f));
   const float z = fmul(s, s);
   float q = ffma(z, kQ9, kQ7);
@@ -88,7 +91,6 @@ __device__ __forceinline__ float log_pos(float u) {
   q = ffma(z, q, kQ3);
   q = ffma(z, q, 1.0f);
   const float lnm = fmul(fmul(2.0f, s), q);
-  const float fe = __int2float_rn(e);
   return ffma(fe, kLn2Hi, ffma(fe, kLn2Lo, lnm));
 }
 
@@ -608,12 +610,13 @@ __device__ __forceinline__ void fold_store(const StreamDev& s, uint32_t* idx, in
 // inputs were loaded ahead, else loaded here). KM >= K: the capacity of the
 // preloaded inputs (a batched kernel loads for up to 8 slots whatever the
 // stream's K; entries past K are dead code once K is a constant).
-template <int KT, int KM = FoldCap<KT>::value>
+// AHEAD: the caller has tested the band and loaded (pre) or not.
+template <int KT, int KM = FoldCap<KT>::value, bool AHEAD = false>
 __device__ __forceinline__ void record_code(const StreamDev& s, const FrameDev& f, int64_t p,
                                             uint8_t c, const FoldIn<KM>* pre) {
   const int K = KT > 0 ? KT : s.K;
   s.maps[static_cast<int64_t>(f.t & kRingMask) * s.plane + p] = c;
-  if (!folds_now(f, p)) return;
+  if (AHEAD ? pre == nullptr : !folds_now(f, p)) return;
   if (pre != nullptr) {
     fold_store(s, s.idx, K, f.t, f.map_lo, p, *pre, c);
   } else {
