@@ -152,9 +152,7 @@ __device__ __forceinline__ int reproject_keys(const StreamDev& cur, const Stream
     if constexpr (F16) {
       const uint2 v = *reinterpret_cast<const uint2*>(sRec + j * kRecStride);
       a = slot_weight_f16(v.y, sWt[j * kThreads] >> lo_shift);
-      cr = __half2float(__ushort_as_half(static_cast<unsigned short>(v.x & 0xffffu)));
-      cg = __half2float(__ushort_as_half(static_cast<unsigned short>(v.x >> 16)));
-      cb = __half2float(__ushort_as_half(static_cast<unsigned short>(v.y & 0xffffu)));
+      slot_colour_f16(v, cr, cg, cb);
     } else {
       const float4 v = *reinterpret_cast<const float4*>(sRec + j * kRecStride);
       a = v.x; cr = v.y; cg = v.z; cb = v.w;
