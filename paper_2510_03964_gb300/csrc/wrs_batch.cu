@@ -4,8 +4,8 @@
 // The launch's descriptor (every stream's planes, frame, gaze, frame index and
 // first tile) travels by value as the kernel parameter, so a batch needs no
 // device memory of its own. Tiles of T = 256 * PX pixels of all streams are
-// numbered stream after stream and dealt to the persistent CTAs round-robin,
-// which spreads every stream (and so every K) evenly over the CTAs. Each tile
+// numbered stream after stream and taken in that order from the hardware's
+// work queue by the CTAs that fit (request_tile). Each tile
 // goes through the same bulk-copy / uniform / compute pipeline as the
 // single-stream kernel (wrs_async.cuh), with the arithmetic chosen per tile by
 // the stream's K and colour precision; results are bit-identical to pushing

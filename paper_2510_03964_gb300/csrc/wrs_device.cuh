@@ -452,7 +452,7 @@ __device__ __forceinline__ void store_rgb(float* dst, const float (&o)[N][3]) {
 
 // With one or two slots the update writes each sample index straight into
 // idx[j] and the state has no code ring: such kernels are bound by
-// instruction issue, not by DRAM, and at their low replacement rates the
+// instruction issue and latency, not by DRAM, and at their low replacement rates the
 // ring's per-pixel work costs more than the scattered index writes it saves.
 //
 // A kernel's KT: its slot count, 0 for any number, or kUpTo8 for any number up
@@ -478,13 +478,10 @@ __device__ __forceinline__ uint32_t after_code(uint32_t v, int j, uint8_t c, uin
   return c == static_cast<uint8_t>(j) ? fr : v;
 }
 
-// The band of 256-pixel block b: (b + b/16 + b/256) mod 16. The persistent
-// kernels deal tiles to CTAs in arithmetic progressions whose step (the grid,
-// 152 SMs x CTAs per SM) is a multiple of 8 or 16, so a band of b % 16 would
-// give each CTA all of its folds in one frame out of 16 (the slowest CTA then
-// sets the frame's time). Adding the higher base-16 digits makes each CTA's
-// blocks run through every band: with 152 or 304 CTAs no CTA folds more than
-// 1.05 times its share in any frame.
+// The band of 256-pixel block b: (b + b/16 + b/256) mod 16. Any 16 neighbouring
+// blocks hold about one of each band, so the tiles in flight at any time fold
+// at an even rate; the higher base-16 digits keep that so for kernels that
+// deal blocks in steps of a multiple of 16.
 __device__ __forceinline__ uint32_t fold_band(int64_t p) {
   const uint32_t b = static_cast<uint32_t>(p >> 8);
   return (b + (b >> 4) + (b >> 8)) & kRingMask;

@@ -1,7 +1,7 @@
 // Pipelined persistent form of the fused update + resolve (sm_103a).
 //
-// Persistent CTAs (one or more per SM) walk the image in tiles of
-// T = 256 * PX pixels. A copying warp streams the planes a tile needs (frame
+// The CTAs that fit on the GPU take the image's tiles of T = 256 * PX pixels in
+// ascending order from the hardware's work queue (request_tile). A copying warp streams the planes a tile needs (frame
 // RGB, W, P, the K key planes and, for the fused resolve, the K slot records)
 // into a ring of S shared-memory stages with 1-D bulk asynchronous copies
 // (cp.async.bulk) that complete on one transaction-count "full" mbarrier per
@@ -10,8 +10,8 @@
 // instructions a tile) held back the copies: 4K K = 8 FP16 244 -> 238 us, 4K
 // literal rule 73.8 -> 69.7 us, 8-stream FP16 batch 990 -> 932 us when the
 // drawing moved to its own warp. Eight consumer warps compute each
-// landed tile from shared memory with the same per-pixel code as the plain
-// kernel (bit-identical results), write straight to global memory and free
+// landed tile from shared memory with the plain kernel's arithmetic
+// (push_staged: bit-identical results), write straight to global memory and free
 // the stage through its "empty" mbarrier. No block-wide barrier sits inside
 // the loop.
 //

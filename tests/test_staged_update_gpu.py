@@ -71,3 +71,41 @@ def test_any_width_equals_the_plain_kernel(wh, K, rule, fp16):
         assert np.array_equal(x[plane].view(np.uint8), y[plane].view(np.uint8)), plane
     assert a.replacements() == b.replacements()
     assert torch.equal(outs[0].view(torch.int32), outs[1].view(torch.int32))
+
+
+def test_captured_calls_equal_eager_calls():
+    """Early launches and the tile queue inside a captured CUDA graph: foveate,
+    push, push_foveated and a reprojected push, replayed once."""
+    w, h, K = 1280, 720, 4
+    rng = np.random.default_rng(3)
+    img = torch.from_numpy(rng.random((h, w, 3), dtype=np.float32)).cuda()
+    motion = torch.full((h, w, 2), 1.25, device="cuda")
+    outs = []
+    for captured in (False, True):
+        st = wrs.Stream(w, h, K, 60.0, seed=9)
+        st.set_reprojection_buffer()
+        fov = wrs.Foveation(img, (60.0, 150.0, 300.0), filter="bilinear")
+        frame, ring = torch.empty_like(img), torch.empty((h, w), dtype=torch.uint8, device="cuda")
+        out = [torch.empty_like(img) for _ in range(3)]
+
+        def calls():
+            fov.rebuild()
+            fov.frame((600.0, 300.0), out=frame, ring_map=ring)
+            st.push_frame(frame, (600.0, 300.0), out=out[0])
+            st.push_foveated(fov, (620.0, 310.0), out=out[1])
+            st.push_frame_reproject(frame, (600.0, 300.0), motion, out=out[2])
+
+        torch.cuda.synchronize()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                calls()
+            g.replay()
+        else:
+            calls()
+        torch.cuda.synchronize()
+        assert st.check_status() == 0
+        state = st.export_state()
+        outs.append([frame, ring, *out, *(torch.from_numpy(np.ascontiguousarray(state[k]).view(np.uint8)) for k in state)])
+    for a, b in zip(*outs):
+        assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
