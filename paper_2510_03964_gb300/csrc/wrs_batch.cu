@@ -63,9 +63,9 @@ struct wrs_batch {
 
 static int px_slot(int px) { return px == 4 ? 2 : (px == 2 ? 1 : 0); }
 
-static int family_of(const BatchArgs& a) {
+static int family_of(const BatchArgs& a, int n) {
   bool f16 = true, f32 = true;
-  for (int i = 0; i < a.n; ++i) {
+  for (int i = 0; i < n; ++i) {
     f16 = f16 && (a.e[i].code == 0 || a.e[i].code == 1);
     f32 = f32 && (a.e[i].code == 2 || a.e[i].code == 3);
   }
@@ -141,6 +141,34 @@ static int code_of(const wrs_config& c) {
   return f16 ? 4 : 5;
 }
 
+// Batches outside the two families (other slot counts, the literal rule, mixed
+// colours) whose streams have at least this many bytes per push (mean over the
+// batch: frame, output, sums and slots) push each stream with its own kernel,
+// back to back: the general batched kernel lacks the forms for one, two and up
+// to 8 slots, but a launch more per stream costs about 4 us. Eight streams (two
+// each of 4K, VR, 1440 x 1600 and HD), batched kernel and own kernels: literal
+// 551 and 310 us, K = 1 751 and 381, K = 3 939 and 774, K = 6 928 and 818; with
+// an eighth of the pixels K = 1 100 and 80, K = 3 125 and 132, K = 6 127 and 145.
+constexpr int64_t kOwnKernelBytes = 112ll << 20, kOwnKernelBytesFew = 24ll << 20;
+
+// Pushes each stream of a validated batch with its own kernel. A launch that
+// fails leaves its stream and the ones after it as they were.
+static int push_each(int n, wrs_ctx* const* ctxs, const BatchEntry* e, bool fov, int filter, cudaStream_t st) {
+  for (int i = 0; i < n; ++i) {
+    wrs_ctx* x = ctxs[i];
+    const bool f16 = x->cfg.color_fp16 != 0;
+    const int stages = fov && x->pipe_px != 1 ? wrs_default_stages(x->cfg.K, f16, 1) : x->pipe_stages;
+    const cudaError_t err =
+        fov ? wrs_launch_pipe_fov(e[i].s, e[i].f, e[i].fv, filter, f16, stages, x->sms, x->pipe_ctas,
+                                  e[i].status, x->timeout_ns, st)
+            : wrs_launch_pipe(e[i].s, e[i].f, f16, x->pipe_px, stages, x->sms, x->pipe_ctas, e[i].status,
+                              x->timeout_ns, 0u, st);
+    if (err != cudaSuccess) return wrs_cuda_fail(err, "push_batch: launch");
+    x->t += 1;
+  }
+  return WRS_OK;
+}
+
 // Validates and launches one batch; sources == NULL: the frames are in
 // d_frames; else stream i's frame is foveated on read from sources[i] with
 // `filter` (d_frames unused).
@@ -157,7 +185,8 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   // the foveating form takes one pixel per thread (256-pixel tiles)
   const int px = fov ? 1 : b->px;
   const int T = 256 * px;
-  int64_t tiles = 0;
+  int64_t tiles = 0, bytes = 0;
+  int most_slots = 0;
   bool maps = false;
   uint32_t stage_bytes = 0;
   int device = -1;
@@ -210,6 +239,8 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     e.tile0 = static_cast<uint32_t>(tiles);
     e.code = code_of(x->cfg);
     tiles += (static_cast<int64_t>(e.s.hw) + T - 1) / T;
+    if (x->cfg.K > most_slots) most_slots = x->cfg.K;
+    bytes += static_cast<int64_t>(e.s.hw) * (40 + x->cfg.K * (x->cfg.color_fp16 ? 14 : 20));
     const bool records = out != nullptr || x->cfg.temporal_bias == 2;
     const uint32_t sb = wrs::stage_layout(T, x->cfg.K, x->cfg.color_fp16 ? 2 : 4, records,
                                           x->cfg.update_rule == WRS_RULE_LITERAL)
@@ -217,6 +248,9 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     if (sb > stage_bytes) stage_bytes = sb;
   }
   if (tiles > 0x7FFFFFFF) return wrs_fail(WRS_ERR_ARG, "batch too large");
+  if (b->px == 1 && b->stages == 0 && b->ctas_per_sm == 0 && family_of(a, n) == kFamAll &&
+      bytes >= (most_slots <= 2 ? kOwnKernelBytesFew : kOwnKernelBytes) * n)
+    return push_each(n, ctxs, a.e, fov, filter, static_cast<cudaStream_t>(stream));
   int stages = b->stages;
   if (stages == 0) {
     // as many stages (up to 4) as keep two CTAs on an SM, else what one CTA holds
@@ -239,7 +273,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   a.stage_bytes = stage_bytes;
   a.timeout_ns = ctxs[0]->timeout_ns;
 
-  const int fam = family_of(a);
+  const int fam = family_of(a, n);
   const int slot = fov ? 9 + fam * 2 + filter : px_slot(px) * 3 + fam;
   const void* fn = fov ? wrs_batch_fov_kernel(fam, filter) : batch_kernel_for(px, fam);
   cudaError_t e = cudaSuccess;

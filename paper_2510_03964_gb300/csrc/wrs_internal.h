@@ -60,6 +60,7 @@ cudaError_t wrs_launch_pipe(const wrs::StreamDev& s, const wrs::FrameDev& f, boo
                             int stages, int sms, int ctas_per_sm, uint32_t* status,
                             uint64_t timeout_ns, uint32_t extra_tx, cudaStream_t st);
 void wrs_default_pipe(int K, bool f16, int* px, int* stages);
+int wrs_default_stages(int K, bool f16, int px);
 
 void wrs_clear_error();
 // WRS_OK, or WRS_ERR_STATE (with the message set) if the context's reservoirs are undefined.

@@ -155,7 +155,7 @@ uint32_t* wrs_status_word(const wrs_ctx* x) {
 // Stages of `px` pixels per thread: as many (up to four) as keep two CTAs on
 // an SM, else what one CTA holds. More stages keep more bytes in flight; the
 // kernels wait on copies, not on arithmetic.
-static int wrs_default_stages(int K, bool f16, int px) {
+int wrs_default_stages(int K, bool f16, int px) {
   constexpr size_t kSmPerSm = 228 * 1024, kReservedPerCta = 1024;
   int st = 4;
   while (st > 2 && 2 * (wrs_pipe_smem_bytes(K, f16, px, st, true) + kReservedPerCta) > kSmPerSm) --st;
