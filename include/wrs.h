@@ -320,9 +320,12 @@ int wrs_checked_build(void);
 /* A batch launcher: pushes one frame into each of up to max_streams streams
  * (any mix of sizes, K and colour precision, all on one device) with a single
  * persistent launch. The launch is a kernel node of a CUDA graph, built on
- * the first push and updated in place for every later push. The library owns
- * the launcher and its graphs (host objects and driver handles only: no
- * device memory). */
+ * the first push and updated in place for every later push. With the default
+ * launch shape, batches that are neither all FP16 nor all FP32 with K = 4 or 8
+ * and whose streams are large (their bytes per push, on average: 24 MiB with
+ * up to two slots each, else 112 MiB) launch each stream's own kernel back to
+ * back instead, which is faster there. The library owns the launcher and its
+ * graphs (host objects and driver handles only: no device memory). */
 typedef struct wrs_batch wrs_batch;
 int wrs_batch_create(int max_streams, wrs_batch** out);
 int wrs_batch_destroy(wrs_batch* batch);
@@ -344,7 +347,8 @@ int wrs_batch_get_launch(const wrs_batch* batch, int* px_per_thread, int* stages
  * may appear once per batch. gaze_xy is host memory. Each stream's state and
  * output are bit-identical to pushing it alone. Every stream's frame counter
  * advances. Errors: WRS_ERR_ARG, WRS_ERR_STATE, WRS_ERR_CUDA (nothing is
- * launched on error). */
+ * launched on error; only where each stream has its own launch and the driver
+ * refuses one of them, the streams before it have advanced). */
 int wrs_push_batch(wrs_batch* batch, int n, wrs_ctx* const* ctxs, const float* const* d_frames,
                    const float* gaze_xy, const uint8_t* const* d_fov_maps, float* const* d_outs,
                    wrs_stream_t stream);
