@@ -109,3 +109,38 @@ def test_captured_calls_equal_eager_calls():
         outs.append([frame, ring, *out, *(torch.from_numpy(np.ascontiguousarray(state[k]).view(np.uint8)) for k in state)])
     for a, b in zip(*outs):
         assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+
+
+@pytest.mark.parametrize("foveated", [False, True])
+@pytest.mark.parametrize("w,h,K,rule,fp16", [(1024, 516, 1, 1, True), (1024, 512, 1, 0, False), (1280, 772, 6, 0, True),
+                                             (1600, 1028, 3, 0, False)])
+def test_large_general_batches_equal_the_batched_kernel(w, h, K, rule, fp16, foveated):
+    """Batches outside the K = 4 / 8 families whose streams are large enough for
+    their own kernels (default launch shape) against the batched kernel (an
+    explicit shape): mixed biases, a flush map and a missing output."""
+    rng = np.random.default_rng(w + K)
+    runs = []
+    for shape in (None, (1, 1, 0, True)):
+        streams = [wrs.Stream(w, h, K, 80.0, seed=4, stream_id=i, color_fp16=fp16, update_rule=rule,
+                              temporal_bias=i % 3) for i in range(3)]
+        b = wrs.Batch(3)
+        if shape:
+            b.set_launch(*shape)
+        runs.append((streams, b, [torch.zeros((h, w, 3), device="cuda") for _ in range(3)]))
+    for t in range(4):
+        frames = [torch.from_numpy(rng.random((h, w, 3), dtype=np.float32)).cuda() for _ in range(3)]
+        fov = torch.from_numpy(rng.choice(np.uint8([0, 255]), (h, w), p=[0.95, 0.05])).cuda()
+        gazes = [(100.0 * i + t, 50.0 * i) for i in range(3)]
+        sources = [wrs.Foveation(f, (80.0, 200.0, 400.0), filter="bilinear") for f in frames] if foveated else frames
+        for streams, b, outs in runs:
+            push = b.push_foveated if foveated else b.push
+            push(streams, sources, gazes, fov_maps=[None, fov, None], outs=[outs[0], outs[1], None])
+    for i in range(3):
+        a, c = runs[0][0][i], runs[1][0][i]
+        assert a.check_status() == 0 and c.check_status() == 0
+        assert a.frame_index == c.frame_index == 4
+        x, y = a.export_state(), c.export_state()
+        for plane in x:
+            assert np.array_equal(x[plane].view(np.uint8), y[plane].view(np.uint8)), (i, plane)
+        assert a.replacements() == c.replacements()
+        assert torch.equal(runs[0][2][i].view(torch.int32), runs[1][2][i].view(torch.int32))
