@@ -320,8 +320,9 @@ __device__ __forceinline__ void add_warp_count(unsigned long long* total, int co
 // instead of ending after its own tile, cancels a CTA that has not started and
 // takes its tile, in ascending order. A fixed deal (tile it * grid + CTA) let
 // CTAs near the memory run ahead; the tiles in flight then spread over the
-// planes, and at 4K K = 8 FP16 the same 1.5 GB of traffic took 267 us where
-// tiles handed out in order take 237 (FP32: 279 and 274).
+// planes, and at 4K K = 8 FP16 the same 1.5 GB of traffic took 250 to 267 us,
+// depending on the box, where tiles handed out in order take 224 (FP32: 275 and
+// 267).
 
 // Asks for the tile of a CTA that has not started: 16 bytes to `resp`,
 // completing 16 transactions on `bar`. One thread; at most one request in

@@ -184,8 +184,8 @@ __device__ __forceinline__ void blend_quad(const float4* row0, const float4* row
 // level's borders read each texel column once (four columns at level 1, three
 // at level 2, two beyond, where x0 % 4 == 0 puts the columns' borders between
 // fixed pixels) with their fractions known, and blend two channels per
-// instruction. 4K, three radii: the kernel takes 33 us instead of
-// 35 alone.
+// instruction: 320 instructions per quad, and 4K with three radii takes 31.5 us
+// instead of 35 under the profiler, 29.2 instead of 36.6 back to back.
 // Returns the four levels, one per byte.
 template <int FILTER>
 __device__ __forceinline__ uint32_t fov_quad(const FovDev& a, float gx, float gy, int32_t x0,
