@@ -47,11 +47,13 @@ struct BatchArgs {
 // kernel parameters may take up to 32764 bytes on sm_70 and later (CUDA 12.1+)
 static_assert(sizeof(BatchArgs) <= 32000, "batch descriptor too large for a kernel parameter");
 
-// The entry (stream) of global tile g: the last entry with tile0 <= g. A CTA
-// visits its tiles in ascending order, so each of its warps keeps the entry of
-// its previous tile in `e` and moves it forward (a few steps per stream
-// boundary instead of a search per tile).
-__device__ __forceinline__ int entry_after(const BatchArgs& a, uint32_t g, int e) {
+// The entry (stream) of global tile g: the last entry with tile0 <= g, searched
+// from the entry `e` of the warp's previous tile. The work queue hands tiles
+// out in ascending order (a few steps per stream boundary instead of a search
+// per tile), but its contract only names some tile not yet taken, so a lower
+// one is looked for as well.
+__host__ __device__ __forceinline__ int entry_of(const BatchArgs& a, uint32_t g, int e) {
+  while (e > 0 && a.e[e].tile0 > g) --e;
   while (e + 1 < a.n && a.e[e + 1].tile0 <= g) ++e;
   return e;
 }
@@ -133,7 +135,7 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
     int pe = 0;  // entry of the copying warp's current tile
     issued = wrs::produce<true>(r, a.timeout_ns, lane,
                                 [&](uint32_t g, uint8_t* st, float*, uint64_t* full, int ln) {
-      pe = entry_after(a, g, pe);
+      pe = entry_of(a, g, pe);
       const BatchEntry& e = a.e[pe];
       const int64_t p0 = static_cast<int64_t>(g - e.tile0) * T;
       constexpr bool cf = FOVF < 0;
@@ -151,7 +153,7 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
     int pe = 0;
     wrs::produce<false>(r, a.timeout_ns, lane,
                         [&](uint32_t g, uint8_t*, float* u, uint64_t* full, int ln) {
-      pe = entry_after(a, g, pe);
+      pe = entry_of(a, g, pe);
       const BatchEntry& e = a.e[pe];
       wrs::draw_tile<T>(e.s, e.f, static_cast<int64_t>(g - e.tile0) * T, u, full, ln);
     });
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
     if constexpr (FOVF >= 0)
       wrs::produce<false>(r, a.timeout_ns, lane,
                           [&](uint32_t g, uint8_t* st, float*, uint64_t* full, int ln) {
-        pe = entry_after(a, g, pe);
+        pe = entry_of(a, g, pe);
         const BatchEntry& e = a.e[pe];
         wrs::foveate_tile<FOVF>(e.s, e.f, e.fv, g - e.tile0, st, full, warp - kConsumerWarps - 2, ln);
       });
@@ -169,7 +171,7 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
     int ei = 0;        // entry of the consumer's current tile
     int replaced = 0;  // this thread's replacements in entry ei so far
     wrs::consume(r, a.timeout_ns, lane, [&](uint32_t g) {
-      const int next = entry_after(a, g, ei);
+      const int next = entry_of(a, g, ei);
       if (next != ei) {
         flush_count(replaced_s, ei, replaced, lane);
         ei = next;

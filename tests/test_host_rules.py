@@ -1,0 +1,46 @@
+"""Rules that the kernels and the host share, compiled for the host and run there (no GPU)."""
+import ctypes as C
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2510_03964_gb300 import build
+
+SRC = r"""
+#include "wrs_batch_kernel.cuh"
+
+extern "C" void entries(int n, const unsigned* tile0, int tiles, const unsigned* order, int* entry) {
+  BatchArgs* a = new BatchArgs();
+  a->n = n;
+  for (int i = 0; i < n; ++i) a->e[i].tile0 = tile0[i];
+  int e = 0;
+  for (int i = 0; i < tiles; ++i) entry[i] = e = entry_of(*a, order[i], e);
+  delete a;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    (d / "rules.cu").write_text(SRC)
+    subprocess.run([build.nvcc(), *build.ARCH, *build.NVCC_FLAGS, "-O1", "-shared", "-cudart", "static",
+                    "-o", str(d / "librules.so"), str(d / "rules.cu")], check=True)
+    return C.CDLL(str(d / "librules.so"))
+
+
+@pytest.mark.parametrize("order", ["ascending", "descending", "shuffled"])
+@pytest.mark.parametrize("sizes", [[1], [5, 1, 1, 7], [1, 300, 2, 2, 40, 1], [3] * 64])
+def test_tile_entries_in_any_order(lib, sizes, order):
+    """The work queue names a tile that no CTA has taken; which one is not part of its contract."""
+    tile0 = np.cumsum([0] + sizes[:-1]).astype(np.uint32)
+    tiles = np.arange(sum(sizes), dtype=np.uint32)
+    if order == "descending":
+        tiles = tiles[::-1].copy()
+    elif order == "shuffled":
+        np.random.default_rng(7).shuffle(tiles)
+    got = np.full(tiles.size, -1, np.int32)
+    lib.entries(len(sizes), tile0.ctypes.data_as(C.c_void_p), tiles.size, tiles.ctypes.data_as(C.c_void_p),
+                got.ctypes.data_as(C.c_void_p))
+    assert np.array_equal(got, np.repeat(np.arange(len(sizes)), sizes)[tiles])
