@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kMipThreads) mip_kernel(MipArgs a) {
     if (VEC && y < a.height && left >= 4) {
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(src) + i);
+        const float4 t = reinterpret_cast<const float4*>(src)[i];
         v[r][4 * i] = t.x;
         v[r][4 * i + 1] = t.y;
         v[r][4 * i + 2] = t.z;
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kMipThreads) mip_kernel(MipArgs a) {
       // pixels outside the image count as 0
       const int in_row = y < a.height ? 3 * (left < 4 ? left : 4) : 0;
 #pragma unroll
-      for (int i = 0; i < 12; ++i) v[r][i] = i < in_row ? __ldg(src + i) : 0.0f;
+      for (int i = 0; i < 12; ++i) v[r][i] = i < in_row ? src[i] : 0.0f;
     }
   }
 

@@ -14,7 +14,9 @@ namespace wrs {
 // the SMs that the previous kernel of the stream has left and sets up its
 // barriers there; grid_begin then waits until that kernel has completed and its writes
 // are visible. Nothing before grid_begin touches global memory, and every CTA
-// calls it.
+// calls it. A kernel that calls it reads with ordinary loads: what the previous
+// kernel writes changes while this one runs, and the compiler may move a
+// non-coherent load (__ldg) across the wait.
 __device__ __forceinline__ void grid_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -76,13 +78,13 @@ __device__ __forceinline__ void level_colour(const FovDev& a, int L, int32_t x, 
                                              float* rgb) {
   if (L == 0) {
     const float* s = a.img + (int64_t)y * a.pitch + 3 * (int64_t)x;
-    rgb[0] = __ldg(s);
-    rgb[1] = __ldg(s + 1);
-    rgb[2] = __ldg(s + 2);
+    rgb[0] = s[0];
+    rgb[1] = s[1];
+    rgb[2] = s[2];
   } else {
     const MipLevelDev lv = a.lev[L];
     if (FILTER == WRS_FILTER_BOX) {
-      const float4 t = __ldg(lv.texels + (int64_t)(y >> L) * lv.wb + (x >> L));
+      const float4 t = lv.texels[(int64_t)(y >> L) * lv.wb + (x >> L)];
       rgb[0] = t.x;
       rgb[1] = t.y;
       rgb[2] = t.z;
@@ -91,10 +93,10 @@ __device__ __forceinline__ void level_colour(const FovDev& a, int L, int32_t x, 
       float fx, fy;
       texel_coord(x, L, lv.wb, &x0, &x1, &fx);
       texel_coord(y, L, lv.hb, &y0, &y1, &fy);
-      const float4 t00 = __ldg(lv.texels + (int64_t)y0 * lv.wb + x0);
-      const float4 t01 = __ldg(lv.texels + (int64_t)y0 * lv.wb + x1);
-      const float4 t10 = __ldg(lv.texels + (int64_t)y1 * lv.wb + x0);
-      const float4 t11 = __ldg(lv.texels + (int64_t)y1 * lv.wb + x1);
+      const float4 t00 = lv.texels[(int64_t)y0 * lv.wb + x0];
+      const float4 t01 = lv.texels[(int64_t)y0 * lv.wb + x1];
+      const float4 t10 = lv.texels[(int64_t)y1 * lv.wb + x0];
+      const float4 t11 = lv.texels[(int64_t)y1 * lv.wb + x1];
       const float gx_ = __fsub_rn(1.0f, fx), gy_ = __fsub_rn(1.0f, fy);
       rgb[0] = lerp2(lerp2(t00.x, t01.x, gx_, fx), lerp2(t10.x, t11.x, gx_, fx), gy_, fy);
       rgb[1] = lerp2(lerp2(t00.y, t01.y, gx_, fx), lerp2(t10.y, t11.y, gx_, fx), gy_, fy);
@@ -142,7 +144,7 @@ struct Texel {
   uint64_t rg, b0;
 };
 __device__ __forceinline__ Texel load_texel(const float4* t) {
-  const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(t));
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(t);
   return {v.x, v.y};
 }
 
@@ -201,7 +203,7 @@ __device__ __forceinline__ uint32_t fov_quad(const FovDev& a, float gx, float gy
       if (((reinterpret_cast<uintptr_t>(a.img) | (uintptr_t)(4 * a.pitch)) & 15u) == 0) {
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-          const float4 v = __ldg(reinterpret_cast<const float4*>(s) + i);
+          const float4 v = reinterpret_cast<const float4*>(s)[i];
           rgb[4 * i] = v.x;
           rgb[4 * i + 1] = v.y;
           rgb[4 * i + 2] = v.z;
@@ -209,7 +211,7 @@ __device__ __forceinline__ uint32_t fov_quad(const FovDev& a, float gx, float gy
         }
       } else {
 #pragma unroll
-        for (int i = 0; i < 12; ++i) rgb[i] = __ldg(s + i);
+        for (int i = 0; i < 12; ++i) rgb[i] = s[i];
       }
       return 0u;
     }
@@ -217,7 +219,7 @@ __device__ __forceinline__ uint32_t fov_quad(const FovDev& a, float gx, float gy
     const MipLevelDev lv = a.lev[l];
     if (FILTER == WRS_FILTER_BOX) {
       const float4* row = lv.texels + (int64_t)(y >> l) * lv.wb + (x0 >> l);
-      const float4 t = __ldg(row), u = l == 1 ? __ldg(row + 1) : t;
+      const float4 t = row[0], u = l == 1 ? row[1] : t;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float4 c = i < 2 ? t : u;

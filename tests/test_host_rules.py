@@ -1,5 +1,8 @@
 """Rules that the kernels and the host share, compiled for the host and run there (no GPU)."""
 import ctypes as C
+import glob
+import os
+import re
 import subprocess
 
 import numpy as np
@@ -44,3 +47,15 @@ def test_tile_entries_in_any_order(lib, sizes, order):
     lib.entries(len(sizes), tile0.ctypes.data_as(C.c_void_p), tiles.size, tiles.ctypes.data_as(C.c_void_p),
                 got.ctypes.data_as(C.c_void_p))
     assert np.array_equal(got, np.repeat(np.arange(len(sizes)), sizes)[tiles])
+
+
+def test_no_noncoherent_loads():
+    """Kernels that start before the previous one of their stream has ended (grid_begin) read what
+    that kernel writes: a load through the read-only path may pass the wait, and needs memory that
+    stays as it is for as long as the kernel runs."""
+    early = 0
+    for path in glob.glob(os.path.join(build.CSRC, "*.cu*")):
+        code = re.sub(r"/\*.*?\*/|//[^\n]*", "", open(path).read(), flags=re.S)
+        early += len(re.findall(r"\bgrid_begin\(\);", code))
+        assert not re.findall(r"__ldg\b|\bld\.global[\w.]*\.nc\b|\bconst\s+[\w:]+\s*\*\s*(?:const\s+)?__restrict__", code), path
+    assert early >= 5
