@@ -187,6 +187,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   const int T = 256 * px;
   int64_t tiles = 0, bytes = 0;
   int most_slots = 0;
+  uint32_t extra_tx = 0;
   bool maps = false;
   uint32_t stage_bytes = 0;
   int device = -1;
@@ -240,6 +241,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     e.code = code_of(x->cfg);
     tiles += (static_cast<int64_t>(e.s.hw) + T - 1) / T;
     if (x->cfg.K > most_slots) most_slots = x->cfg.K;
+    if (x->test_extra_tx > extra_tx) extra_tx = x->test_extra_tx;
     bytes += static_cast<int64_t>(e.s.hw) * (40 + x->cfg.K * (x->cfg.color_fp16 ? 14 : 20));
     const bool records = out != nullptr || x->cfg.temporal_bias == 2;
     const uint32_t sb = wrs::stage_layout(T, x->cfg.K, x->cfg.color_fp16 ? 2 : 4, records,
@@ -272,6 +274,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   a.maps = maps ? 1 : 0;
   a.stage_bytes = stage_bytes;
   a.timeout_ns = ctxs[0]->timeout_ns;
+  a.extra_tx = extra_tx;
 
   const int fam = family_of(a, n);
   const int slot = fov ? 9 + fam * 2 + filter : px_slot(px) * 3 + fam;

@@ -42,6 +42,7 @@ struct BatchArgs {
   int stages;
   uint32_t stage_bytes;  // largest stage of any stream in the batch
   uint64_t timeout_ns;
+  uint32_t extra_tx;     // added to the expected bytes: > 0 only to test the timeout path
   BatchEntry e[kMaxBatch];
 };
 // kernel parameters may take up to 32764 bytes on sm_70 and later (CUDA 12.1+)
@@ -94,12 +95,14 @@ __device__ __forceinline__ int tile(const BatchEntry& e, uint8_t* st, const floa
 // K = 4 / 8 families), so the copy sizes and stage offsets fold to constants.
 template <int T, int KT, int CS, bool COPY_FRAME>
 __device__ __forceinline__ void produce_tile(const BatchEntry& e, int64_t p0, uint8_t* st,
-                                             uint64_t* full, int ln, uint32_t stage_cap) {
+                                             uint64_t* full, int ln, uint32_t stage_cap,
+                                             uint32_t extra_tx) {
   const int K = KT > 0 ? KT : e.s.K;
   const int cs = CS > 0 ? CS : (entry_f16(e) ? 2 : 4);
   const bool resolve = stage_records(e);
   const StageLayout L = wrs::stage_layout(T, K, cs, resolve, KT == 0 && e.s.literal != 0);
-  wrs::issue_tile_copies<T, false>(e.s, e.f, K, cs, resolve, L, st, full, p0, 0u, ln, COPY_FRAME, stage_cap);
+  wrs::issue_tile_copies<T, false>(e.s, e.f, K, cs, resolve, L, st, full, p0, extra_tx, ln, COPY_FRAME,
+                                   stage_cap);
 }
 
 // Warp-specialised like the single-stream pipelined kernel: warp 8 issues each
@@ -122,13 +125,18 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
   if (warp == 0) wrs::init_ring(r, kConsumerWarps, batch_producers(FOVF >= 0), lane);
   if (tid < kMaxBatch) replaced_s[tid] = 0;
   // each stream's Eq. (phat) normaliser, once per CTA instead of once per tile
+  bool usable = false;
   if (tid < a.n) {
     d_f_s[tid] = wrs::fovea_density(a.e[tid].s);
     // a stream whose earlier push timed out (not yet seen by the host) has
     // undefined reservoirs: its tiles are copied but not computed or written
-    failed_s[tid] = *reinterpret_cast<volatile const uint32_t*>(a.e[tid].status);
+    const uint32_t failed = *reinterpret_cast<volatile const uint32_t*>(a.e[tid].status);
+    failed_s[tid] = failed;
+    usable = failed == 0;
   }
-  __syncthreads();
+  // nothing to compute: among others the CTAs that start after a wait of this
+  // launch has given up, which then add no waits of their own
+  if (!__syncthreads_or(usable)) return;
 
   int issued = 0;
   if (warp == kConsumerWarps) {
@@ -140,13 +148,13 @@ __global__ void __launch_bounds__(batch_threads(FOVF >= 0), PX == 1 ? 2 : 1)
       const int64_t p0 = static_cast<int64_t>(g - e.tile0) * T;
       constexpr bool cf = FOVF < 0;
       if constexpr (FAM == kFamF16K48) {
-        if (e.code == 0) produce_tile<T, 4, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
-        else produce_tile<T, 8, 2, cf>(e, p0, st, full, ln, r.stage_bytes);
+        if (e.code == 0) produce_tile<T, 4, 2, cf>(e, p0, st, full, ln, r.stage_bytes, a.extra_tx);
+        else produce_tile<T, 8, 2, cf>(e, p0, st, full, ln, r.stage_bytes, a.extra_tx);
       } else if constexpr (FAM == kFamF32K48) {
-        if (e.code == 2) produce_tile<T, 4, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
-        else produce_tile<T, 8, 4, cf>(e, p0, st, full, ln, r.stage_bytes);
+        if (e.code == 2) produce_tile<T, 4, 4, cf>(e, p0, st, full, ln, r.stage_bytes, a.extra_tx);
+        else produce_tile<T, 8, 4, cf>(e, p0, st, full, ln, r.stage_bytes, a.extra_tx);
       } else {
-        produce_tile<T, 0, 0, cf>(e, p0, st, full, ln, r.stage_bytes);
+        produce_tile<T, 0, 0, cf>(e, p0, st, full, ln, r.stage_bytes, a.extra_tx);
       }
     });
   } else if (warp == kConsumerWarps + 1) {

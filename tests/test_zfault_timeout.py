@@ -86,3 +86,37 @@ def test_timed_out_push_is_refused_until_a_saved_state_is_restored():
     torch.cuda.synchronize()
     assert st.check_status() == WRS_OK
     run.compare()
+
+
+@pytest.mark.parametrize("K", [4, 3])
+def test_timed_out_batch_ends_soon_and_recovers(K):
+    """A batch of many more tiles than CTAs that fit: once a wait has given up, the CTAs that
+    start later add no waits of their own. A CTA spends at most a limit in its loops, one on an
+    answer of the queue and one per stage while its copies land (six with four stages); the
+    8,192 tiles are 13 times the CTAs that fit or more."""
+    import time
+    limit = 0.02
+    sts = [wrs.Stream(1024, 1024, K, 50.0, seed=2, stream_id=i) for i in range(2)]
+    frames = [torch.rand((1024, 1024, 3), device="cuda") for _ in sts]
+    gazes = [(500.0, 300.0)] * 2
+    b = wrs.Batch(2)
+    b.push(sts, frames, gazes)
+    assert all(st.check_status() == WRS_OK for st in sts)
+    snaps = [st.export_raw() for st in sts]
+    for st in sts:
+        st.set_wait_limit(timeout_ns=int(limit * 1e9), test_extra_tx=16)
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    b.push(sts, frames, gazes)
+    torch.cuda.synchronize()
+    assert time.perf_counter() - t0 < 2 * 6 * limit
+    for st, snap in zip(sts, snaps):
+        assert st.check_status() == WRS_ERR_TIMEOUT
+        st.set_wait_limit(0, 0)
+        st.import_raw(snap, 1)
+    b.push(sts, frames, gazes)
+    solo = wrs.Stream(1024, 1024, K, 50.0, seed=2, stream_id=1)
+    for _ in range(2):
+        solo.push_frame(frames[1], gazes[1])
+    assert all(st.check_status() == WRS_OK for st in sts)
+    assert np.array_equal(sts[1].export_raw()[256:], solo.export_raw()[256:])
