@@ -36,7 +36,8 @@ constexpr uint64_t kDefaultTimeoutNs = 2000000000ull;  // 2 s
 constexpr size_t kSmemBudget = 227 * 1024 - 1024;       // dynamic shared memory per CTA we use
 
 // Launches a kernel that calls wrs::grid_begin: it may start before the
-// previous kernel of the stream has ended.
+// previous kernel of the stream has ended. A refusal is the caller's to report
+// and leaves no error that a later launch would read as its own.
 template <typename... P, typename... A>
 cudaError_t wrs_launch_early(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
                              cudaStream_t st, const A&... args) {
@@ -50,7 +51,9 @@ cudaError_t wrs_launch_early(void (*kernel)(P...), dim3 grid, int threads, size_
   how.stream = st;
   how.attrs = &early;
   how.numAttrs = 1;
-  return cudaLaunchKernelEx(&how, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&how, kernel, args...);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
 }
 
 uint32_t* wrs_status_word(const wrs_ctx* x);

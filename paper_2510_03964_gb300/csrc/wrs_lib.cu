@@ -36,6 +36,7 @@ void wrs_clear_error() { g_err[0] = '\0'; }
 extern "C" const char* wrs_last_error(void) { return g_err; }
 
 int wrs_cuda_fail(cudaError_t e, const char* what) {
+  (void)cudaGetLastError();  // reported here: a later launch must not read it as its own
   return wrs_fail(WRS_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 

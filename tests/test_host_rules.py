@@ -12,6 +12,7 @@ from paper_2510_03964_gb300 import build
 
 SRC = r"""
 #include "wrs_batch_kernel.cuh"
+#include "wrs_internal.h"
 
 extern "C" void entries(int n, const unsigned* tile0, int tiles, const unsigned* order, int* entry) {
   BatchArgs* a = new BatchArgs();
@@ -20,6 +21,16 @@ extern "C" void entries(int n, const unsigned* tile0, int tiles, const unsigned*
   int e = 0;
   for (int i = 0; i < tiles; ++i) entry[i] = e = entry_of(*a, order[i], e);
   delete a;
+}
+
+__global__ void nothing(int) {}
+
+// a launch that the runtime refuses (more threads than a block can have), then
+// the error that the next launch's cudaGetLastError would report
+extern "C" void refused(int* refusal, int* left) {
+  (void)cudaGetLastError();
+  *refusal = wrs_launch_early(nothing, dim3(1), 4096, 0, nullptr, 0);
+  *left = cudaGetLastError();
 }
 """
 
@@ -47,6 +58,14 @@ def test_tile_entries_in_any_order(lib, sizes, order):
     lib.entries(len(sizes), tile0.ctypes.data_as(C.c_void_p), tiles.size, tiles.ctypes.data_as(C.c_void_p),
                 got.ctypes.data_as(C.c_void_p))
     assert np.array_equal(got, np.repeat(np.arange(len(sizes)), sizes)[tiles])
+
+
+def test_a_refused_launch_leaves_no_error_behind(lib):
+    """The next launch of the thread must not be taken for refused: the host would not count a
+    frame that the device has pushed."""
+    refusal, left = C.c_int(0), C.c_int(-1)
+    lib.refused(C.byref(refusal), C.byref(left))
+    assert refusal.value != 0 and left.value == 0
 
 
 def test_no_noncoherent_loads():
