@@ -11,6 +11,22 @@ import pytest
 from paper_2510_03964_gb300 import build
 
 SRC = r"""
+#include <cuda_runtime.h>
+
+// a runtime that refuses every launch, with the last-error state of the real one
+static cudaError_t g_last = cudaSuccess;
+static cudaError_t last_error() {
+  const cudaError_t e = g_last;
+  g_last = cudaSuccess;
+  return e;
+}
+template <typename... T>
+cudaError_t refuse(const T&...) {
+  return g_last = cudaErrorInvalidConfiguration;
+}
+#define cudaGetLastError last_error
+#define cudaLaunchKernelEx refuse
+
 #include "wrs_batch_kernel.cuh"
 #include "wrs_internal.h"
 
@@ -25,12 +41,10 @@ extern "C" void entries(int n, const unsigned* tile0, int tiles, const unsigned*
 
 __global__ void nothing(int) {}
 
-// a launch that the runtime refuses (more threads than a block can have), then
-// the error that the next launch's cudaGetLastError would report
+// a refused launch, then what the next launch's cudaGetLastError would report
 extern "C" void refused(int* refusal, int* left) {
-  (void)cudaGetLastError();
-  *refusal = wrs_launch_early(nothing, dim3(1), 4096, 0, nullptr, 0);
-  *left = cudaGetLastError();
+  *refusal = wrs_launch_early(nothing, dim3(1), 32, 0, nullptr, 0);
+  *left = last_error();
 }
 """
 
