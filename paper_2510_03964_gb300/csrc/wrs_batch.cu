@@ -157,11 +157,12 @@ static int push_each(int n, wrs_ctx* const* ctxs, const BatchEntry* e, bool fov,
   for (int i = 0; i < n; ++i) {
     wrs_ctx* x = ctxs[i];
     const bool f16 = x->cfg.color_fp16 != 0;
-    const int stages = fov && x->pipe_px != 1 ? wrs_default_stages(x->cfg.K, f16, 1) : x->pipe_stages;
+    int px, stages;
+    wrs_pipe_shape(x, fov, &px, &stages);
     const cudaError_t err =
         fov ? wrs_launch_pipe_fov(e[i].s, e[i].f, e[i].fv, filter, f16, stages, x->sms, x->pipe_ctas,
                                   e[i].status, x->timeout_ns, st)
-            : wrs_launch_pipe(e[i].s, e[i].f, f16, x->pipe_px, stages, x->sms, x->pipe_ctas, e[i].status,
+            : wrs_launch_pipe(e[i].s, e[i].f, f16, px, stages, x->sms, x->pipe_ctas, e[i].status,
                               x->timeout_ns, 0u, st);
     if (err != cudaSuccess) return wrs_cuda_fail(err, "push_batch: launch");
     x->t += 1;

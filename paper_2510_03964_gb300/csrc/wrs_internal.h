@@ -64,6 +64,11 @@ cudaError_t wrs_launch_pipe(const wrs::StreamDev& s, const wrs::FrameDev& f, boo
                             uint64_t timeout_ns, uint32_t extra_tx, cudaStream_t st);
 void wrs_default_pipe(int K, bool f16, int* px, int* stages);
 int wrs_default_stages(int K, bool f16, int px);
+// Pixels per thread and stages of a pipelined push of the stream: as set, or
+// the default stages where the push takes one pixel per thread (one_px) and
+// another number was set, or the default shape where what was set does not fit
+// (wrs_set_pipeline checks that only when it enables the pipelined kernel).
+void wrs_pipe_shape(const wrs_ctx* x, bool one_px, int* px, int* stages);
 
 void wrs_clear_error();
 // WRS_OK, or WRS_ERR_STATE (with the message set) if the context's reservoirs are undefined.

@@ -173,6 +173,18 @@ void wrs_default_pipe(int K, bool f16, int* px, int* stages) {
   *stages = wrs_default_stages(K, f16, *px);
 }
 
+void wrs_pipe_shape(const wrs_ctx* x, bool one_px, int* px, int* stages) {
+  const bool f16 = x->cfg.color_fp16 != 0;
+  *px = x->pipe_px;
+  *stages = x->pipe_stages;
+  if (!x->pipe && wrs_pipe_smem_bytes(x->cfg.K, f16, *px, *stages, true) > kSmemBudget)
+    wrs_default_pipe(x->cfg.K, f16, px, stages);
+  if (one_px && *px != 1) {
+    *px = 1;
+    *stages = wrs_default_stages(x->cfg.K, f16, 1);
+  }
+}
+
 extern "C" size_t wrs_state_bytes(const wrs_config* cfg) {
   if (wrs_check_config(cfg) != WRS_OK) return 0;
   wrs_layout L;
@@ -458,11 +470,8 @@ extern "C" int wrs_push_frame(wrs_ctx* x, const float* d_frame, int64_t pitch, f
   f.map_lo = wrs_map_lo(x);
   cudaError_t e;
   if (x->pipe && wrs_pipe_supported(x, d_frame, pitch, d_out)) {
-    int px = x->pipe_px, stages = x->pipe_stages;
-    if (px != 1 && x->cfg.width % 4 != 0) {
-      px = 1;  // a thread's pixels lie in one row: see wrs_pipe_supported
-      stages = wrs_default_stages(x->cfg.K, x->cfg.color_fp16 != 0, 1);
-    }
+    int px, stages;
+    wrs_pipe_shape(x, x->cfg.width % 4 != 0, &px, &stages);  // a thread's pixels lie in one row
     e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, px, stages, x->sms, x->pipe_ctas,
                         wrs_status_word(x), x->timeout_ns, x->test_extra_tx,
                         static_cast<cudaStream_t>(stream));
@@ -504,9 +513,8 @@ extern "C" int wrs_push_foveated(wrs_ctx* x, const float* d_img, int64_t img_pit
   f.gy = gy;
   f.t = x->t;
   f.map_lo = wrs_map_lo(x);
-  int px = x->pipe_px, stages = x->pipe_stages;
-  // the foveating form takes one pixel per thread: its own stage count then
-  if (px != 1) stages = wrs_default_stages(x->cfg.K, x->cfg.color_fp16 != 0, 1);
+  int px, stages;
+  wrs_pipe_shape(x, true, &px, &stages);  // the foveating form takes one pixel per thread
   cudaError_t e = wrs_launch_pipe_fov(s, f, fv, filter, x->cfg.color_fp16 != 0, stages, x->sms, x->pipe_ctas,
                                       wrs_status_word(x), x->timeout_ns,
                                       static_cast<cudaStream_t>(stream));

@@ -144,3 +144,24 @@ def test_large_general_batches_equal_the_batched_kernel(w, h, K, rule, fp16, fov
             assert np.array_equal(x[plane].view(np.uint8), y[plane].view(np.uint8)), (i, plane)
         assert a.replacements() == c.replacements()
         assert torch.equal(runs[0][2][i].view(torch.int32), runs[1][2][i].view(torch.int32))
+
+
+def test_large_general_batches_take_streams_with_a_disabled_pipeline():
+    """A shape set with the pipelined kernel disabled is not checked against shared memory; the
+    batch, which always pipelines, takes the stream all the same."""
+    w, h = 1024, 516
+    shapes = [(True, 0, 0, 0), (False, 4, 8, 1), (False, 0, 0, 0)]
+    streams = [wrs.Stream(w, h, 1, 80.0, seed=4, stream_id=i, update_rule=1) for i in range(3)]
+    solo = [wrs.Stream(w, h, 1, 80.0, seed=4, stream_id=i, update_rule=1) for i in range(3)]
+    for st, shape in zip(streams, shapes):
+        st.set_pipeline(*shape)
+    b = wrs.Batch(3)
+    frames = [torch.rand((h, w, 3), device="cuda") for _ in range(3)]
+    outs = [torch.empty_like(f) for f in frames]
+    for t in range(2):
+        b.push(streams, frames, [(100.0, 50.0 * t)] * 3, outs=outs)
+        for st, f in zip(solo, frames):
+            st.push_frame(f, (100.0, 50.0 * t))
+    for a, c in zip(streams, solo):
+        assert a.check_status() == 0 and a.frame_index == 2
+        assert np.array_equal(a.export_raw()[256:], c.export_raw()[256:])
