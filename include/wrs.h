@@ -323,17 +323,20 @@ int wrs_checked_build(void);
  * the first push and updated in place for every later push. With the default
  * launch shape, batches that are neither all FP16 nor all FP32 with K = 4 or 8
  * and whose streams are large (their bytes per push, on average: 24 MiB with
- * up to two slots each, else 112 MiB) launch each stream's own kernel back to
- * back instead, which is faster there. The library owns the launcher and its
- * graphs (host objects and driver handles only: no device memory). */
+ * up to two slots each, else 112 MiB) launch a graph of each stream's own
+ * kernels, one after another, instead, which is faster there (a single such
+ * stream is launched without a graph). The library owns the launcher and its graphs (host objects
+ * and driver handles only: no device memory). */
 typedef struct wrs_batch wrs_batch;
 int wrs_batch_create(int max_streams, wrs_batch** out);
 int wrs_batch_destroy(wrs_batch* batch);
 
 /* Tile and launch shape: tiles of 256 * px_per_thread pixels (1, 2 or 4),
- * `stages` shared-memory stages (0: two, or one if two do not fit),
- * ctas_per_sm persistent CTAs per SM (0: as many as fit), use_graph = 0 for a
- * plain launch instead of the graph. Chosen by the autotuner. */
+ * `stages` shared-memory stages (0: as many, up to four, as keep two CTAs on
+ * an SM, else as many as one CTA holds), ctas_per_sm persistent CTAs per SM (0:
+ * as many as fit), use_graph = 0 for a plain launch instead of the graph. The
+ * default is 1, 0, 0, 1; any other shape always takes the batched kernel.
+ * Chosen by the autotuner. */
 int wrs_batch_set_launch(wrs_batch* batch, int px_per_thread, int stages, int ctas_per_sm,
                          int use_graph);
 int wrs_batch_get_launch(const wrs_batch* batch, int* px_per_thread, int* stages,
@@ -347,8 +350,7 @@ int wrs_batch_get_launch(const wrs_batch* batch, int* px_per_thread, int* stages
  * may appear once per batch. gaze_xy is host memory. Each stream's state and
  * output are bit-identical to pushing it alone. Every stream's frame counter
  * advances. Errors: WRS_ERR_ARG, WRS_ERR_STATE, WRS_ERR_CUDA (nothing is
- * launched on error; only where each stream has its own launch and the driver
- * refuses one of them, the streams before it have advanced). */
+ * launched on error). */
 int wrs_push_batch(wrs_batch* batch, int n, wrs_ctx* const* ctxs, const float* const* d_frames,
                    const float* gaze_xy, const uint8_t* const* d_fov_maps, float* const* d_outs,
                    wrs_stream_t stream);

@@ -19,6 +19,7 @@
 #include "wrs.h"
 #include "wrs_batch_kernel.cuh"
 #include "wrs_internal.h"
+#include "wrs_own.h"
 
 namespace {
 
@@ -57,6 +58,7 @@ struct wrs_batch {
   cudaGraphExec_t exec[kSlots];
   cudaGraphNode_t node[kSlots];
   size_t configured_smem[kSlots];
+  wrs_own own;
   int device;
   int rebuilds;  // graph nodes rebuilt because an in-place update was refused
 };
@@ -98,6 +100,7 @@ extern "C" int wrs_batch_create(int max_streams, wrs_batch** out) {
 
 extern "C" int wrs_batch_destroy(wrs_batch* b) {
   if (!b) return WRS_OK;
+  wrs_own_drop(&b->own);
   for (int i = 0; i < kSlots; ++i) {
     if (b->exec[i]) cudaGraphExecDestroy(b->exec[i]);
     if (b->graph[i]) cudaGraphDestroy(b->graph[i]);
@@ -141,35 +144,6 @@ static int code_of(const wrs_config& c) {
   return f16 ? 4 : 5;
 }
 
-// Batches outside the two families (other slot counts, the literal rule, mixed
-// colours) whose streams have at least this many bytes per push (mean over the
-// batch: frame, output, sums and slots) push each stream with its own kernel,
-// back to back: the general batched kernel lacks the forms for one, two and up
-// to 8 slots, but a launch more per stream costs about 4 us. Eight streams (two
-// each of 4K, VR, 1440 x 1600 and HD), batched kernel and own kernels: literal
-// 551 and 310 us, K = 1 751 and 381, K = 3 939 and 774, K = 6 928 and 818; with
-// an eighth of the pixels K = 1 100 and 80, K = 3 125 and 132, K = 6 127 and 145.
-constexpr int64_t kOwnKernelBytes = 112ll << 20, kOwnKernelBytesFew = 24ll << 20;
-
-// Pushes each stream of a validated batch with its own kernel. A launch that
-// fails leaves its stream and the ones after it as they were.
-static int push_each(int n, wrs_ctx* const* ctxs, const BatchEntry* e, bool fov, int filter, cudaStream_t st) {
-  for (int i = 0; i < n; ++i) {
-    wrs_ctx* x = ctxs[i];
-    const bool f16 = x->cfg.color_fp16 != 0;
-    int px, stages;
-    wrs_pipe_shape(x, fov, &px, &stages);
-    const cudaError_t err =
-        fov ? wrs_launch_pipe_fov(e[i].s, e[i].f, e[i].fv, filter, f16, stages, x->sms, x->pipe_ctas,
-                                  e[i].status, x->timeout_ns, st)
-            : wrs_launch_pipe(e[i].s, e[i].f, f16, px, stages, x->sms, x->pipe_ctas, e[i].status,
-                              x->timeout_ns, 0u, st);
-    if (err != cudaSuccess) return wrs_cuda_fail(err, "push_batch: launch");
-    x->t += 1;
-  }
-  return WRS_OK;
-}
-
 // Validates and launches one batch; sources == NULL: the frames are in
 // d_frames; else stream i's frame is foveated on read from sources[i] with
 // `filter` (d_frames unused).
@@ -186,8 +160,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   // the foveating form takes one pixel per thread (256-pixel tiles)
   const int px = fov ? 1 : b->px;
   const int T = 256 * px;
-  int64_t tiles = 0, bytes = 0;
-  int most_slots = 0;
+  int64_t tiles = 0;
   uint32_t extra_tx = 0;
   bool maps = false;
   uint32_t stage_bytes = 0;
@@ -241,9 +214,7 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     e.tile0 = static_cast<uint32_t>(tiles);
     e.code = code_of(x->cfg);
     tiles += (static_cast<int64_t>(e.s.hw) + T - 1) / T;
-    if (x->cfg.K > most_slots) most_slots = x->cfg.K;
     if (x->test_extra_tx > extra_tx) extra_tx = x->test_extra_tx;
-    bytes += static_cast<int64_t>(e.s.hw) * (40 + x->cfg.K * (x->cfg.color_fp16 ? 14 : 20));
     const bool records = out != nullptr || x->cfg.temporal_bias == 2;
     const uint32_t sb = wrs::stage_layout(T, x->cfg.K, x->cfg.color_fp16 ? 2 : 4, records,
                                           x->cfg.update_rule == WRS_RULE_LITERAL)
@@ -251,13 +222,22 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
     if (sb > stage_bytes) stage_bytes = sb;
   }
   if (tiles > 0x7FFFFFFF) return wrs_fail(WRS_ERR_ARG, "batch too large");
-  if (b->px == 1 && b->stages == 0 && b->ctas_per_sm == 0 && family_of(a, n) == kFamAll &&
-      bytes >= (most_slots <= 2 ? kOwnKernelBytesFew : kOwnKernelBytes) * n)
-    return push_each(n, ctxs, a.e, fov, filter, static_cast<cudaStream_t>(stream));
+  if (b->device != device) {
+    // a new device: drop graphs and attribute settings made for another one
+    for (int i = 0; i < kSlots; ++i) {
+      if (b->exec[i]) cudaGraphExecDestroy(b->exec[i]);
+      if (b->graph[i]) cudaGraphDestroy(b->graph[i]);
+      b->exec[i] = nullptr;
+      b->graph[i] = nullptr;
+      b->configured_smem[i] = 0;
+    }
+    wrs_own_drop(&b->own);
+    b->device = device;
+  }
+  constexpr size_t kSmPerSm = 228 * 1024, kReservedPerCta = 1024;
   int stages = b->stages;
   if (stages == 0) {
     // as many stages (up to 4) as keep two CTAs on an SM, else what one CTA holds
-    constexpr size_t kSmPerSm = 228 * 1024, kReservedPerCta = 1024;
     stages = 4;
     while (stages > 2 && 2 * (wrs::ring_bytes(stage_bytes, T, stages, false) + kReservedPerCta) > kSmPerSm)
       --stages;
@@ -266,6 +246,9 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   size_t smem = wrs::ring_bytes(stage_bytes, T, stages, false);
   if (smem > kSmemBudget)
     return wrs_fail(WRS_ERR_ARG, "%d stages of %u B exceed shared memory", stages, stage_bytes);
+  const bool default_shape = b->px == 1 && b->stages == 0 && b->ctas_per_sm == 0 && b->use_graph;
+  if (default_shape && family_of(a, n) == kFamAll && wrs_own_faster(n, ctxs))
+    return wrs_own_push(&b->own, n, ctxs, a.e, fov, filter, static_cast<cudaStream_t>(stream));
   if (maps) {
     stages = wrs::stages_with_maps(stage_bytes, T, stages);
     smem = wrs::ring_bytes(stage_bytes, T, stages, true);
@@ -281,17 +264,6 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   const int slot = fov ? 9 + fam * 2 + filter : px_slot(px) * 3 + fam;
   const void* fn = fov ? wrs_batch_fov_kernel(fam, filter) : batch_kernel_for(px, fam);
   cudaError_t e = cudaSuccess;
-  if (b->device != device) {
-    // a new device: drop graphs and attribute settings made for another one
-    for (int i = 0; i < kSlots; ++i) {
-      if (b->exec[i]) cudaGraphExecDestroy(b->exec[i]);
-      if (b->graph[i]) cudaGraphDestroy(b->graph[i]);
-      b->exec[i] = nullptr;
-      b->graph[i] = nullptr;
-      b->configured_smem[i] = 0;
-    }
-    b->device = device;
-  }
   if (b->configured_smem[slot] == 0) {
     // allow the whole budget once, before any graph is built: a graph keeps the
     // limit it was instantiated under, and later batches may need larger stages

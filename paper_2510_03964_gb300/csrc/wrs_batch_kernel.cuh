@@ -15,10 +15,7 @@ using wrs::FrameDev;
 using wrs::StageLayout;
 using wrs::StreamDev;
 
-namespace {
-
-constexpr int kMaxBatch = WRS_MAX_BATCH;
-
+// One stream of a batch and its frame.
 struct BatchEntry {
   StreamDev s;
   FrameDev f;
@@ -28,6 +25,10 @@ struct BatchEntry {
   int code;    // arithmetic variant: 0 K=4 f16, 1 K=8 f16, 2 K=4 f32, 3 K=8 f32, 4 any K f16,
                // 5 any K f32, 6 literal f16, 7 literal f32
 };
+
+namespace {
+
+constexpr int kMaxBatch = WRS_MAX_BATCH;
 
 // The slot records are staged when the fused resolve needs them or the full
 // temporal bias forms the history's resolved colour from them.

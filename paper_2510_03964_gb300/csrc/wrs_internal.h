@@ -38,9 +38,8 @@ constexpr size_t kSmemBudget = 227 * 1024 - 1024;       // dynamic shared memory
 // Launches a kernel that calls wrs::grid_begin: it may start before the
 // previous kernel of the stream has ended. A refusal is the caller's to report
 // and leaves no error that a later launch would read as its own.
-template <typename... P, typename... A>
-cudaError_t wrs_launch_early(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
-                             cudaStream_t st, const A&... args) {
+inline cudaError_t wrs_launch_early_params(const void* kernel, dim3 grid, int threads, size_t smem,
+                                           cudaStream_t st, void** params) {
   cudaLaunchAttribute early;
   early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   early.val.programmaticStreamSerializationAllowed = 1;
@@ -51,17 +50,50 @@ cudaError_t wrs_launch_early(void (*kernel)(P...), dim3 grid, int threads, size_
   how.stream = st;
   how.attrs = &early;
   how.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&how, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelExC(&how, kernel, params);
   if (e != cudaSuccess) (void)cudaGetLastError();
   return e;
+}
+template <typename... P>
+cudaError_t wrs_launch_early(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                             cudaStream_t st, const P&... args) {
+  void* params[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  return wrs_launch_early_params(reinterpret_cast<const void*>(kernel), grid, threads, smem, st, params);
 }
 
 uint32_t* wrs_status_word(const wrs_ctx* x);
 size_t wrs_pipe_smem_bytes(int K, bool f16, int px, int stages, bool resolve);
 bool wrs_pipe_supported(const wrs_ctx* x, const float* frame, int64_t pitch, const float* out);
-cudaError_t wrs_launch_pipe(const wrs::StreamDev& s, const wrs::FrameDev& f, bool f16, int px,
-                            int stages, int sms, int ctas_per_sm, uint32_t* status,
-                            uint64_t timeout_ns, uint32_t extra_tx, cudaStream_t st);
+
+// Arguments of the pipelined kernel beside the stream, the frame and the source.
+struct wrs_pipe_args {
+  int stages;
+  int queue;               // more tiles than CTAs that fit: see Ring::queue
+  int resolve;             // copy weight/colour planes (fused resolve or full temporal bias)
+  uint32_t* status;        // stream status word (WRS_OK or WRS_ERR_TIMEOUT)
+  uint64_t timeout_ns;
+  uint32_t extra_tx;       // added to the expected bytes: > 0 only to test the timeout path
+};
+// A pipelined push that only has to be launched: everything the runtime could
+// refuse about its shape has been asked. `params` point into the plan and at
+// the stream, frame and source it was made for, which have to outlive the launch call.
+struct wrs_pipe_plan {
+  const void* fn;
+  unsigned grid;
+  int threads;
+  size_t smem;
+  wrs_pipe_args a;
+  void* params[4];
+};
+cudaError_t wrs_plan_pipe(const wrs::StreamDev& s, const wrs::FrameDev& f, bool f16, int px,
+                          int stages, int sms, int ctas_per_sm, uint32_t* status,
+                          uint64_t timeout_ns, uint32_t extra_tx, wrs_pipe_plan* plan);
+// The pipelined kernel foveating the frame as it reads it (filter: WRS_FILTER_*).
+cudaError_t wrs_plan_pipe_fov(const wrs::StreamDev& s, const wrs::FrameDev& f,
+                              const wrs::FovDev& fv, int filter, bool f16, int stages, int sms,
+                              int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
+                              uint32_t extra_tx, wrs_pipe_plan* plan);
+cudaError_t wrs_launch_plan(const wrs_pipe_plan& plan, cudaStream_t st);
 void wrs_default_pipe(int K, bool f16, int* px, int* stages);
 int wrs_default_stages(int K, bool f16, int px);
 // Pixels per thread and stages of a pipelined push of the stream: as set, or
@@ -90,10 +122,5 @@ int wrs_effective_px(const wrs_ctx* x, const float* frame, int64_t pitch, const 
 int wrs_fov_check_source(const float* d_img, int64_t pitch, const void* d_mip, size_t mip_bytes,
                    int32_t width, int32_t height, int32_t nradii, const float* radii,
                    int32_t filter, wrs::FovDev* fv);
-// The pipelined kernel foveating the frame as it reads it (filter: WRS_FILTER_*).
-cudaError_t wrs_launch_pipe_fov(const wrs::StreamDev& s, const wrs::FrameDev& f,
-                                const wrs::FovDev& fv, int filter, bool f16, int stages, int sms,
-                                int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
-                                cudaStream_t st);
 cudaError_t wrs_launch_push(const wrs::StreamDev& s, const wrs::FrameDev& f, int block, int px,
                             bool f16, cudaStream_t st);

@@ -472,9 +472,10 @@ extern "C" int wrs_push_frame(wrs_ctx* x, const float* d_frame, int64_t pitch, f
   if (x->pipe && wrs_pipe_supported(x, d_frame, pitch, d_out)) {
     int px, stages;
     wrs_pipe_shape(x, x->cfg.width % 4 != 0, &px, &stages);  // a thread's pixels lie in one row
-    e = wrs_launch_pipe(s, f, x->cfg.color_fp16 != 0, px, stages, x->sms, x->pipe_ctas,
-                        wrs_status_word(x), x->timeout_ns, x->test_extra_tx,
-                        static_cast<cudaStream_t>(stream));
+    wrs_pipe_plan plan;
+    e = wrs_plan_pipe(s, f, x->cfg.color_fp16 != 0, px, stages, x->sms, x->pipe_ctas,
+                      wrs_status_word(x), x->timeout_ns, x->test_extra_tx, &plan);
+    if (e == cudaSuccess) e = wrs_launch_plan(plan, static_cast<cudaStream_t>(stream));
   } else {
     const int px = wrs_effective_px(x, d_frame, pitch, d_out);
     e = wrs_launch_push(s, f, x->block, px, x->cfg.color_fp16 != 0,
@@ -515,9 +516,10 @@ extern "C" int wrs_push_foveated(wrs_ctx* x, const float* d_img, int64_t img_pit
   f.map_lo = wrs_map_lo(x);
   int px, stages;
   wrs_pipe_shape(x, true, &px, &stages);  // the foveating form takes one pixel per thread
-  cudaError_t e = wrs_launch_pipe_fov(s, f, fv, filter, x->cfg.color_fp16 != 0, stages, x->sms, x->pipe_ctas,
-                                      wrs_status_word(x), x->timeout_ns,
-                                      static_cast<cudaStream_t>(stream));
+  wrs_pipe_plan plan;
+  cudaError_t e = wrs_plan_pipe_fov(s, f, fv, filter, x->cfg.color_fp16 != 0, stages, x->sms,
+                                    x->pipe_ctas, wrs_status_word(x), x->timeout_ns, 0u, &plan);
+  if (e == cudaSuccess) e = wrs_launch_plan(plan, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return wrs_cuda_fail(e, "wrs_push_foveated: launch");
   x->t += 1;
   return WRS_OK;

@@ -35,14 +35,7 @@ using wrs::StreamDev;
 
 namespace {
 
-struct PipeArgs {
-  int stages;
-  int queue;               // more tiles than CTAs that fit: see Ring::queue
-  int resolve;             // copy weight/colour planes (fused resolve or full temporal bias)
-  uint32_t* status;        // stream status word (WRS_OK or WRS_ERR_TIMEOUT)
-  uint64_t timeout_ns;
-  uint32_t extra_tx;       // added to the expected bytes: > 0 only to test the timeout path
-};
+using PipeArgs = wrs_pipe_args;
 
 constexpr int kConsumerWarps = 8;
 // FOVF >= 0: the frame is not copied but foveated from `fv` with filter FOVF
@@ -137,9 +130,11 @@ __global__ void __launch_bounds__(pipe_threads(FOVF), pipe_min_blocks<KT, PX, LI
   }
 }
 
+const FovDev kNoSource{};
+
 template <int KT, bool F16, int PX, bool LIT = false, int FOVF = -1>
-cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int sms, int ctas_per_sm,
-                          cudaStream_t st, const FovDev& fv = FovDev{}) {
+cudaError_t plan_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int sms, int ctas_per_sm,
+                        wrs_pipe_plan* plan, const FovDev& fv = kNoSource) {
   constexpr int T = kConsumerWarps * 32 * PX;
   const StageLayout L = wrs::stage_layout(T, s.K, F16 ? 2 : 4, a.resolve != 0, LIT);
   if (f.fov != nullptr) a.stages = wrs::stages_with_maps(L.bytes, T, a.stages);
@@ -180,48 +175,57 @@ cudaError_t launch_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int
   }
   const int64_t tiles = (static_cast<int64_t>(s.hw) + T - 1) / T;
   a.queue = tiles > static_cast<int64_t>(fit) * sms ? 1 : 0;
-  return wrs_launch_early(kernel, dim3(static_cast<unsigned>(tiles)), pipe_threads(FOVF), smem, st, s, f, a, fv);
+  plan->fn = reinterpret_cast<const void*>(kernel);
+  plan->grid = static_cast<unsigned>(tiles);
+  plan->threads = pipe_threads(FOVF);
+  plan->smem = smem;
+  plan->a = a;
+  plan->params[0] = const_cast<StreamDev*>(&s);
+  plan->params[1] = const_cast<FrameDev*>(&f);
+  plan->params[2] = &plan->a;
+  plan->params[3] = const_cast<FovDev*>(&fv);
+  return cudaSuccess;
 }
 
 // The foveating form: one pixel per thread (the default tile), K = 4, 8 or
 // any other through the generic instantiation, and the literal rule.
 template <bool F16, int FILTER>
-cudaError_t launch_pipe_fov_k(const StreamDev& s, const FrameDev& f, const FovDev& fv,
-                              const PipeArgs& a, int sms, int ctas, cudaStream_t st) {
-  if (s.literal) return launch_pipe_t<1, F16, 1, true, FILTER>(s, f, a, sms, ctas, st, fv);
+cudaError_t plan_pipe_fov_k(const StreamDev& s, const FrameDev& f, const FovDev& fv,
+                              const PipeArgs& a, int sms, int ctas, wrs_pipe_plan* plan) {
+  if (s.literal) return plan_pipe_t<1, F16, 1, true, FILTER>(s, f, a, sms, ctas, plan, fv);
   switch (s.K) {
-    case 4: return launch_pipe_t<4, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
-    case 8: return launch_pipe_t<8, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
+    case 4: return plan_pipe_t<4, F16, 1, false, FILTER>(s, f, a, sms, ctas, plan, fv);
+    case 8: return plan_pipe_t<8, F16, 1, false, FILTER>(s, f, a, sms, ctas, plan, fv);
     default:
-      if (s.K <= 8) return launch_pipe_t<wrs::kUpTo8, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
-      return launch_pipe_t<0, F16, 1, false, FILTER>(s, f, a, sms, ctas, st, fv);
+      if (s.K <= 8) return plan_pipe_t<wrs::kUpTo8, F16, 1, false, FILTER>(s, f, a, sms, ctas, plan, fv);
+      return plan_pipe_t<0, F16, 1, false, FILTER>(s, f, a, sms, ctas, plan, fv);
   }
 }
 
 template <int KT, bool F16, bool LIT = false>
-cudaError_t launch_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
-                            cudaStream_t st) {
+cudaError_t plan_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
+                            wrs_pipe_plan* plan) {
   switch (px) {
-    case 4: return launch_pipe_t<KT, F16, 4, LIT>(s, f, a, sms, ctas, st);
-    case 2: return launch_pipe_t<KT, F16, 2, LIT>(s, f, a, sms, ctas, st);
-    default: return launch_pipe_t<KT, F16, 1, LIT>(s, f, a, sms, ctas, st);
+    case 4: return plan_pipe_t<KT, F16, 4, LIT>(s, f, a, sms, ctas, plan);
+    case 2: return plan_pipe_t<KT, F16, 2, LIT>(s, f, a, sms, ctas, plan);
+    default: return plan_pipe_t<KT, F16, 1, LIT>(s, f, a, sms, ctas, plan);
   }
 }
 
 template <bool F16>
-cudaError_t launch_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
-                           cudaStream_t st) {
-  if (s.literal) return launch_pipe_px<1, F16, true>(s, f, a, px, sms, ctas, st);
+cudaError_t plan_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
+                           wrs_pipe_plan* plan) {
+  if (s.literal) return plan_pipe_px<1, F16, true>(s, f, a, px, sms, ctas, plan);
   switch (s.K) {
-    case 1: return launch_pipe_px<1, F16>(s, f, a, px, sms, ctas, st);
-    case 2: return launch_pipe_px<2, F16>(s, f, a, px, sms, ctas, st);
-    case 4: return launch_pipe_px<4, F16>(s, f, a, px, sms, ctas, st);
-    case 8: return launch_pipe_px<8, F16>(s, f, a, px, sms, ctas, st);
+    case 1: return plan_pipe_px<1, F16>(s, f, a, px, sms, ctas, plan);
+    case 2: return plan_pipe_px<2, F16>(s, f, a, px, sms, ctas, plan);
+    case 4: return plan_pipe_px<4, F16>(s, f, a, px, sms, ctas, plan);
+    case 8: return plan_pipe_px<8, F16>(s, f, a, px, sms, ctas, plan);
     default:
       // other slot counts: up to 8 unrolled with a test per slot, 9 to 16
       // through run-time loops (184 x 143, K = 6: 4.8 us against 10.6)
-      if (px == 1 && s.K <= 8) return launch_pipe_t<wrs::kUpTo8, F16, 1>(s, f, a, sms, ctas, st);
-      return launch_pipe_px<0, F16>(s, f, a, px, sms, ctas, st);
+      if (px == 1 && s.K <= 8) return plan_pipe_t<wrs::kUpTo8, F16, 1>(s, f, a, sms, ctas, plan);
+      return plan_pipe_px<0, F16>(s, f, a, px, sms, ctas, plan);
   }
 }
 
@@ -243,31 +247,36 @@ bool wrs_pipe_supported(const wrs_ctx* x, const float* frame, int64_t pitch, con
   return pitch == 3 * static_cast<int64_t>(x->cfg.width) && al(frame) && (out == nullptr || al(out));
 }
 
-cudaError_t wrs_launch_pipe_fov(const StreamDev& s, const FrameDev& f, const FovDev& fv, int filter,
+cudaError_t wrs_plan_pipe_fov(const StreamDev& s, const FrameDev& f, const FovDev& fv, int filter,
                                 bool f16, int stages, int sms, int ctas_per_sm, uint32_t* status,
-                                uint64_t timeout_ns, cudaStream_t st) {
-  PipeArgs a;
-  a.stages = stages;
-  a.resolve = (f.out != nullptr || s.bias == 2) ? 1 : 0;  // records: resolve or Delta L
-  a.status = status;
-  a.timeout_ns = timeout_ns;
-  a.extra_tx = 0;
-  if (filter == WRS_FILTER_BOX)
-    return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, st)
-               : launch_pipe_fov_k<false, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, st);
-  return f16 ? launch_pipe_fov_k<true, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, st)
-             : launch_pipe_fov_k<false, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, st);
-}
-
-cudaError_t wrs_launch_pipe(const StreamDev& s, const FrameDev& f, bool f16, int px, int stages,
-                            int sms, int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
-                            uint32_t extra_tx, cudaStream_t st) {
+                                uint64_t timeout_ns, uint32_t extra_tx, wrs_pipe_plan* plan) {
   PipeArgs a;
   a.stages = stages;
   a.resolve = (f.out != nullptr || s.bias == 2) ? 1 : 0;  // records: resolve or Delta L
   a.status = status;
   a.timeout_ns = timeout_ns;
   a.extra_tx = extra_tx;
-  return f16 ? launch_pipe_k<true>(s, f, a, px, sms, ctas_per_sm, st)
-             : launch_pipe_k<false>(s, f, a, px, sms, ctas_per_sm, st);
+  if (filter == WRS_FILTER_BOX)
+    return f16 ? plan_pipe_fov_k<true, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, plan)
+               : plan_pipe_fov_k<false, WRS_FILTER_BOX>(s, f, fv, a, sms, ctas_per_sm, plan);
+  return f16 ? plan_pipe_fov_k<true, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, plan)
+             : plan_pipe_fov_k<false, WRS_FILTER_BILINEAR>(s, f, fv, a, sms, ctas_per_sm, plan);
+}
+
+cudaError_t wrs_plan_pipe(const StreamDev& s, const FrameDev& f, bool f16, int px, int stages,
+                            int sms, int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
+                            uint32_t extra_tx, wrs_pipe_plan* plan) {
+  PipeArgs a;
+  a.stages = stages;
+  a.resolve = (f.out != nullptr || s.bias == 2) ? 1 : 0;  // records: resolve or Delta L
+  a.status = status;
+  a.timeout_ns = timeout_ns;
+  a.extra_tx = extra_tx;
+  return f16 ? plan_pipe_k<true>(s, f, a, px, sms, ctas_per_sm, plan)
+             : plan_pipe_k<false>(s, f, a, px, sms, ctas_per_sm, plan);
+}
+
+cudaError_t wrs_launch_plan(const wrs_pipe_plan& plan, cudaStream_t st) {
+  return wrs_launch_early_params(plan.fn, dim3(plan.grid), plan.threads, plan.smem, st,
+                                 const_cast<void**>(plan.params));
 }

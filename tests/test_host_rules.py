@@ -25,7 +25,7 @@ cudaError_t refuse(const T&...) {
   return g_last = cudaErrorInvalidConfiguration;
 }
 #define cudaGetLastError last_error
-#define cudaLaunchKernelEx refuse
+#define cudaLaunchKernelExC refuse
 
 #include "wrs_batch_kernel.cuh"
 #include "wrs_internal.h"
@@ -48,14 +48,86 @@ extern "C" void refused(int* refusal, int* left) {
 }
 """
 
+OWN = r"""
+#include <cuda_runtime.h>
+
+// a runtime that counts launches of kernels and graphs and refuses one of them
+static int g_launches = 0, g_refused = -1;
+static cudaError_t launch() { return g_launches++ == g_refused ? cudaErrorLaunchFailure : cudaSuccess; }
+template <typename... T>
+cudaError_t fine(const T&...) {
+  return cudaSuccess;
+}
+template <typename... T>
+cudaError_t launch_graph(const T&...) {
+  return launch();
+}
+template <typename... T>
+cudaError_t instantiate(cudaGraphExec_t* exec, const T&...) {
+  *exec = reinterpret_cast<cudaGraphExec_t>(exec);
+  return cudaSuccess;
+}
+#define cudaGetLastError fine
+#define cudaStreamIsCapturing fine
+#define cudaGraphCreate fine
+#define cudaGraphAddKernelNode fine
+#define cudaGraphAddDependencies fine
+#define cudaGraphInstantiate instantiate
+#define cudaGraphExecKernelNodeSetParams fine
+#define cudaGraphExecDestroy fine
+#define cudaGraphDestroy fine
+#define cudaGraphLaunch launch_graph
+
+#include "wrs_own.cu"
+
+int wrs_cuda_fail(cudaError_t, const char*) { return WRS_ERR_CUDA; }
+void wrs_pipe_shape(const wrs_ctx*, bool, int*, int*) {}
+cudaError_t wrs_plan_pipe(const wrs::StreamDev&, const wrs::FrameDev&, bool, int, int, int, int, uint32_t*,
+                          uint64_t, uint32_t, wrs_pipe_plan*) {
+  return cudaSuccess;
+}
+cudaError_t wrs_plan_pipe_fov(const wrs::StreamDev&, const wrs::FrameDev&, const wrs::FovDev&, int, bool, int,
+                              int, int, uint32_t*, uint64_t, uint32_t, wrs_pipe_plan*) {
+  return cudaSuccess;
+}
+cudaError_t wrs_launch_plan(const wrs_pipe_plan&, cudaStream_t) { return launch(); }
+
+// pushes a batch of n streams twice; the launch of that number is refused
+extern "C" int push_twice(int n, int refuse, unsigned* frames) {
+  static wrs_ctx ctx[WRS_MAX_BATCH];
+  static BatchEntry entry[WRS_MAX_BATCH];
+  static wrs_own own;
+  wrs_ctx* ctxs[WRS_MAX_BATCH];
+  own = wrs_own();
+  for (int i = 0; i < n; ++i) {
+    ctx[i] = wrs_ctx();
+    ctxs[i] = &ctx[i];
+  }
+  g_launches = 0;
+  g_refused = refuse;
+  int rc = wrs_own_push(&own, n, ctxs, entry, false, 0, nullptr);
+  if (rc == WRS_OK) rc = wrs_own_push(&own, n, ctxs, entry, false, 0, nullptr);
+  for (int i = 0; i < n; ++i) frames[i] = ctx[i].t;
+  return rc;
+}
+"""
+
+
+def _compile(d, name, source):
+    (d / f"{name}.cu").write_text(source)
+    subprocess.run([build.nvcc(), *build.ARCH, *build.NVCC_FLAGS, "-O1", "-shared", "-cudart", "static",
+                    "-o", str(d / f"{name}.so"), str(d / f"{name}.cu")], check=True)
+    return C.CDLL(str(d / f"{name}.so"))
+
 
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
-    d = tmp_path_factory.mktemp("rules")
-    (d / "rules.cu").write_text(SRC)
-    subprocess.run([build.nvcc(), *build.ARCH, *build.NVCC_FLAGS, "-O1", "-shared", "-cudart", "static",
-                    "-o", str(d / "librules.so"), str(d / "rules.cu")], check=True)
-    return C.CDLL(str(d / "librules.so"))
+    return _compile(tmp_path_factory.mktemp("rules"), "rules", SRC)
+
+
+@pytest.fixture(scope="module")
+def own(tmp_path_factory):
+    return _compile(tmp_path_factory.mktemp("own"), "own", OWN)
 
 
 @pytest.mark.parametrize("order", ["ascending", "descending", "shuffled"])
@@ -92,3 +164,11 @@ def test_no_noncoherent_loads():
         early += len(re.findall(r"\bgrid_begin\(\);", code))
         assert not re.findall(r"__ldg\b|\bld\.global[\w.]*\.nc\b|\bconst\s+[\w:]+\s*\*\s*(?:const\s+)?__restrict__", code), path
     assert early >= 5
+
+
+@pytest.mark.parametrize("n", [1, 2, 8])
+def test_a_batch_through_own_kernels_is_launched_whole_or_not_at_all(own, n):
+    frames = (C.c_uint * n)()
+    assert own.push_twice(n, -1, frames) == 0 and list(frames) == [2] * n
+    for refused in (0, 1):
+        assert own.push_twice(n, refused, frames) != 0 and list(frames) == [refused] * n

@@ -165,3 +165,36 @@ def test_large_general_batches_take_streams_with_a_disabled_pipeline():
     for a, c in zip(streams, solo):
         assert a.check_status() == 0 and a.frame_index == 2
         assert np.array_equal(a.export_raw()[256:], c.export_raw()[256:])
+
+
+@pytest.mark.parametrize("captured", [False, True])
+def test_large_general_batches_of_changing_streams(captured):
+    """Rounds of changing number, order and kind of streams through one launcher (the graph of own
+    kernels is updated or built anew), eagerly and inside a captured graph, against single pushes."""
+    kinds = [(1280, 772, 1, 1, False), (1280, 772, 6, 0, True), (1600, 1028, 3, 0, True), (1024, 512, 16, 0, False)]
+    mixed, solo = ([wrs.Stream(w, h, K, 60.0, seed=8, stream_id=i, color_fp16=f, update_rule=r)
+                    for i, (w, h, K, r, f) in enumerate(kinds)] for _ in range(2))
+    frames = [torch.rand((h, w, 3), device="cuda") for w, h, *_ in kinds]
+    outs, single = ([torch.zeros_like(f) for f in frames] for _ in range(2))
+    b = wrs.Batch(4)
+    for t, members in enumerate(([0, 1, 2], [0, 1, 2], [2, 0, 1], [1, 2], [3, 2, 1, 0], [2], [0, 1, 2])):
+        def push():
+            b.push([mixed[i] for i in members], [frames[i] for i in members],
+                   [(30.0 * t, 40.0 * i) for i in members], outs=[outs[i] for i in members])
+
+        torch.cuda.synchronize()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                push()
+            g.replay()
+            torch.cuda.synchronize()
+        else:
+            push()
+        for i in members:
+            solo[i].push_frame(frames[i], (30.0 * t, 40.0 * i), out=single[i])
+    for i, (a, c) in enumerate(zip(mixed, solo)):
+        assert a.check_status() == 0 and c.check_status() == 0 and a.frame_index == c.frame_index
+        assert a.replacements() == c.replacements()
+        assert np.array_equal(a.export_raw()[256:], c.export_raw()[256:]), i
+        assert torch.equal(outs[i].view(torch.int32), single[i].view(torch.int32)), i
