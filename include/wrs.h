@@ -322,10 +322,10 @@ int wrs_checked_build(void);
  * persistent launch. The launch is a kernel node of a CUDA graph, built on
  * the first push and updated in place for every later push. With the default
  * launch shape, batches that are neither all FP16 nor all FP32 with K = 4 or 8
- * and whose streams are large (their bytes per push, on average: 24 MiB with
- * up to two slots each, else 112 MiB) launch a graph of each stream's own
- * kernels, one after another, instead, which is faster there (a single such
- * stream is launched without a graph). The library owns the launcher and its graphs (host objects
+ * and large enough for their slot counts (a rule fitted to measurements)
+ * launch a graph of each stream's own kernels, one after another, instead:
+ * faster there, with the same results (a single such stream is launched
+ * without a graph). The library owns the launcher and its graphs (host objects
  * and driver handles only: no device memory). */
 typedef struct wrs_batch wrs_batch;
 int wrs_batch_create(int max_streams, wrs_batch** out);

@@ -247,7 +247,8 @@ static int push_batch(wrs_batch* b, int n, wrs_ctx* const* ctxs, const float* co
   if (smem > kSmemBudget)
     return wrs_fail(WRS_ERR_ARG, "%d stages of %u B exceed shared memory", stages, stage_bytes);
   const bool default_shape = b->px == 1 && b->stages == 0 && b->ctas_per_sm == 0 && b->use_graph;
-  if (default_shape && family_of(a, n) == kFamAll && wrs_own_faster(n, ctxs))
+  if (default_shape && family_of(a, n) == kFamAll &&
+      wrs_own_faster(n, ctxs, fov, 2 * (smem + kReservedPerCta) > kSmPerSm))
     return wrs_own_push(&b->own, n, ctxs, a.e, fov, filter, static_cast<cudaStream_t>(stream));
   if (maps) {
     stages = wrs::stages_with_maps(stage_bytes, T, stages);

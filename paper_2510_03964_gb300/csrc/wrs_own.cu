@@ -3,24 +3,42 @@
 
 #include <cstring>
 
-// The streams' bytes per push (mean over the batch: frame, output, sums and
-// slots) from which their own kernels are taken: the general batched kernel
-// lacks the forms for one, two and up to 8 slots, but a kernel more per stream
-// costs about 4 us. Eight streams (two each of 4K, VR, 1440 x 1600 and HD),
-// batched kernel and own kernels: literal 551 and 310 us, K = 1 751 and 381,
-// K = 3 939 and 774, K = 6 928 and 828; with an eighth of the pixels K = 1 100
-// and 80, K = 3 125 and 132, K = 6 127 and 145.
-constexpr int64_t kOwnKernelBytes = 112ll << 20, kOwnKernelBytesFew = 24ll << 20;
+// Microseconds per million pixels that a stream takes longer as a part of the
+// batched kernel for all forms than through its own kernel, which holds one
+// form only (unrolled for its slot count, fold inputs ahead, stages of its own
+// size). Fitted to batches of eight streams (two each of 4K, VR, 1440 x 1600 and
+// HD, of K and min(K, 4) slots, back to back) at 34.5 and 8.3 Mpx in all, for
+// instance, batched and own kernels, us: literal FP16 569 and 295, 145 and 102;
+// K = 3 FP16 953 and 770, 240 and 219; K = 6 FP32 895 and 862, 228 and 247; K = 8
+// and 4 of different colours 895 and 899; foveated K = 6 FP16 1255 and 945.
+static double own_gain(const wrs_config& c, bool fov, bool one_cta) {
+  const bool f16 = c.color_fp16 != 0;
+  if (c.update_rule == WRS_RULE_LITERAL) return fov ? 5.5 : 8.5;
+  if (c.K >= 9) return fov ? 8.0 : 6.0;
+  // own kernels keep two CTAs on an SM where one large stream leaves the
+  // batched kernel one: K = 16 and 4 FP16 2004 and 1499 us
+  const double alone = one_cta ? (fov ? 18.0 : 13.0) : 0.0;
+  switch (c.K) {
+    case 1: return alone + (fov ? 10.0 : 12.0);
+    case 2: return alone + (fov ? 10.0 : f16 ? 10.0 : 9.0);
+    case 3: return alone + (fov ? 11.0 : 6.0);
+    case 4: return alone + (fov ? 8.0 : f16 ? 3.0 : 1.5);
+    case 8: return alone + (fov ? 3.0 : 0.0);
+    default: return alone + (fov ? 12.0 : f16 ? 7.0 : 3.0);
+  }
+}
 
-bool wrs_own_faster(int n, wrs_ctx* const* ctxs) {
-  int64_t bytes = 0;
-  int most_slots = 0;
+bool wrs_own_faster(int n, wrs_ctx* const* ctxs, bool fov, bool one_cta) {
+  double gain = 0.0;
+  bool few = true;
   for (int i = 0; i < n; ++i) {
     const wrs_config& c = ctxs[i]->cfg;
-    if (c.K > most_slots) most_slots = c.K;
-    bytes += static_cast<int64_t>(c.width) * c.height * (40 + c.K * (c.color_fp16 ? 14 : 20));
+    gain += 1e-6 * c.width * static_cast<double>(c.height) * own_gain(c, fov, one_cta);
+    few = few && c.K <= 3;
   }
-  return bytes >= (most_slots <= 2 ? kOwnKernelBytesFew : kOwnKernelBytes) * n;
+  // what each kernel after the first costs: its start and its last tiles (the
+  // same fits; a 4K K = 16 stream and 15 of 256 x 256: 695 us batched, 718)
+  return gain > (n - 1) * (fov ? 6.0 : few ? 4.5 : 5.5);
 }
 
 void wrs_own_drop(wrs_own* o) {

@@ -17,7 +17,9 @@ struct wrs_own {
 
 // Whether a batch outside the batched kernel's two families (other slot counts,
 // the literal rule, mixed colours) is faster through the streams' own kernels.
-bool wrs_own_faster(int n, wrs_ctx* const* ctxs);
+// one_cta: the batched kernel's stages, sized for the largest stream, leave
+// room for one CTA on an SM.
+bool wrs_own_faster(int n, wrs_ctx* const* ctxs, bool fov, bool one_cta);
 // Pushes the validated entries; WRS_OK, or WRS_ERR_CUDA with nothing launched.
 int wrs_own_push(wrs_own* o, int n, wrs_ctx* const* ctxs, const BatchEntry* e, bool fov, int filter,
                  cudaStream_t st);

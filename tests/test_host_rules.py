@@ -110,6 +110,21 @@ extern "C" int push_twice(int n, int refuse, unsigned* frames) {
   for (int i = 0; i < n; ++i) frames[i] = ctx[i].t;
   return rc;
 }
+
+extern "C" int faster(int n, const int* w, const int* h, const int* K, const int* literal, const int* f16, int fov,
+                      int one_cta) {
+  static wrs_ctx ctx[WRS_MAX_BATCH];
+  wrs_ctx* ctxs[WRS_MAX_BATCH];
+  for (int i = 0; i < n; ++i) {
+    ctxs[i] = &ctx[i];
+    ctx[i].cfg.width = w[i];
+    ctx[i].cfg.height = h[i];
+    ctx[i].cfg.K = K[i];
+    ctx[i].cfg.update_rule = literal[i] ? WRS_RULE_LITERAL : WRS_RULE_KEYS;
+    ctx[i].cfg.color_fp16 = f16[i];
+  }
+  return wrs_own_faster(n, ctxs, fov != 0, one_cta != 0);
+}
 """
 
 
@@ -172,3 +187,36 @@ def test_a_batch_through_own_kernels_is_launched_whole_or_not_at_all(own, n):
     assert own.push_twice(n, -1, frames) == 0 and list(frames) == [2] * n
     for refused in (0, 1):
         assert own.push_twice(n, refused, frames) != 0 and list(frames) == [refused] * n
+
+
+def _mix(scale, K, literal=False, f16=True):
+    """Two streams of each size, K and min(K, 4) slots; f16 None: colours mixed."""
+    out = []
+    for w, h in ((3840, 2160), (2064, 2208), (1440, 1600), (1920, 1080)):
+        for i, k in enumerate((K, min(4, K))):
+            out.append((round(w * scale / 4) * 4, round(h * scale), k, literal, f16 if f16 is not None else i == 0))
+    return out
+
+
+@pytest.mark.parametrize("streams,fov,one_cta,faster", [
+    # measured, us: the batched kernel, a graph of own kernels
+    (_mix(1.0, 1, True), 0, 0, True),                # 569, 295
+    (_mix(0.347, 1, True), 0, 0, True),              # 78, 70
+    (_mix(0.245, 1, True), 0, 0, False),             # 43, 47
+    (_mix(0.49, 3), 0, 0, True),                     # 240, 219
+    (_mix(0.347, 3), 0, 0, False),                   # 127, 132
+    (_mix(1.0, 6, f16=False), 0, 0, True),           # 895, 862
+    (_mix(0.49, 6, f16=False), 0, 0, False),         # 228, 247
+    (_mix(0.49, 12), 0, 0, False),                   # 294, 300
+    (_mix(0.347, 16), 0, 1, True),                   # 254, 229
+    (_mix(1.0, 8, f16=None), 0, 0, False),           # 895, 899
+    (_mix(1.0, 8, f16=None), 1, 0, True),            # 1085, 924
+    (_mix(0.347, 1, True), 1, 0, False),             # 123, 130
+    ([(3840, 2160, 16, 0, 1)] + [(256, 256, 16, 0, 1)] * 15, 0, 1, False),  # 695, 718
+    ([(3840, 2160, 1, 1, 1)] + [(256, 256, 1, 1, 1)] * 15, 0, 0, True),     # 160, 130
+    ([(3840, 2160, 1, 1, 1)] + [(256, 256, 1, 1, 1)] * 40, 0, 0, False),    # 191, 231
+    ([(1920, 1080, 3, 0, 1)], 0, 0, True),           # 67, 50
+])
+def test_general_batches_take_the_measured_faster_form(own, streams, fov, one_cta, faster):
+    cols = [(C.c_int * len(streams))(*[int(v) for v in col]) for col in zip(*streams)]
+    assert bool(own.faster(len(streams), *cols, fov, one_cta)) == faster
