@@ -9,8 +9,9 @@ launching stream, and keeps the fastest:
   pixels per thread;
 * batch: the batched kernel's tile, stages, CTAs per SM and graph/plain launch.
 
-Results are cached per device name and shape signature in
-``_build/autotune.json`` next to the library, so the sweep runs once.
+Results are cached per device name, library sources and shape signature in
+``_build/autotune.json`` next to the library, so the sweep runs once and a
+shape found for other kernels is not taken for the present ones.
 Candidates that do not fit (shared memory, registers) are rejected by the
 library itself and skipped here.
 """
@@ -38,7 +39,7 @@ BATCH_CANDIDATES = [(px, st, ctas, g) for px in (1, 2) for st in (0, 2, 3) for c
 
 def _key(kind: str, shapes) -> str:
     name = torch.cuda.get_device_name()
-    return f"{name}|{kind}|" + ";".join(",".join(str(v) for v in s) for s in shapes)
+    return f"{name}|{_build.fingerprint()}|{kind}|" + ";".join(",".join(str(v) for v in s) for s in shapes)
 
 
 def _load_cache() -> dict:

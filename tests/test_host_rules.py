@@ -220,3 +220,16 @@ def _mix(scale, K, literal=False, f16=True):
 def test_general_batches_take_the_measured_faster_form(own, streams, fov, one_cta, faster):
     cols = [(C.c_int * len(streams))(*[int(v) for v in col]) for col in zip(*streams)]
     assert bool(own.faster(len(streams), *cols, fov, one_cta)) == faster
+
+
+def test_a_tuned_launch_shape_belongs_to_the_sources_it_was_tuned_with(tmp_path, monkeypatch):
+    import torch
+    from paper_2510_03964_gb300 import autotune
+    monkeypatch.setattr(torch.cuda, "get_device_name", lambda: "GB300")
+    src = tmp_path / "kernel.cu"
+    src.write_text("// one tile per CTA\n")
+    monkeypatch.setattr(build, "_deps", lambda: [str(src)])
+    keys = [autotune._key("stream", [(64, 32, 4, 0)]), autotune._key("stream", [(64, 32, 4, 0)])]
+    src.write_text("// a fixed deal\n")
+    keys.append(autotune._key("stream", [(64, 32, 4, 0)]))
+    assert keys[0] == keys[1] != keys[2]
