@@ -198,3 +198,39 @@ def test_large_general_batches_of_changing_streams(captured):
         assert a.replacements() == c.replacements()
         assert np.array_equal(a.export_raw()[256:], c.export_raw()[256:]), i
         assert torch.equal(outs[i].view(torch.int32), single[i].view(torch.int32)), i
+
+
+@pytest.mark.parametrize("wh,K,rule,fp16,bias,shape", [
+    ((1365, 767), 1, 1, False, 1, None), ((1365, 767), 4, 0, False, 2, None), ((1365, 767), 6, 0, True, 1, None),
+    ((2064, 1104), 1, 0, True, 2, None), ((2064, 1104), 2, 0, False, 1, None), ((2064, 1104), 4, 0, True, 1, None),
+    ((2064, 1104), 8, 0, True, 2, None), ((2064, 1104), 8, 0, False, 1, None), ((2064, 1104), 3, 0, False, 2, None),
+    ((2064, 1104), 1, 1, True, 2, None), ((1364, 768), 5, 0, False, 1, (1, 1, 1)), ((1364, 768), 8, 0, True, 1, (1, 2, 1)),
+    ((1364, 768), 4, 0, False, 2, (1, 8, 1)), ((2064, 1104), 2, 0, True, 1, (4, 2, 1)), ((2064, 1104), 16, 0, True, 1, None),
+])
+def test_refilled_stages_equal_the_plain_kernel(wh, K, rule, fp16, bias, shape):
+    """Seven to 29 tiles per CTA (152 to 456 CTAs, 256 to 1,024 pixels per tile): the stages are
+    refilled after their columns were written (flushes, rescales, replaced slots), and the queue's
+    answers wrap around. Some colours are infinite, NaN or beyond FP16."""
+    w, h = wh
+    rng = np.random.default_rng(K + 10 * bias)
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    a, b = (wrs.Stream(w, h, K, 60.0, seed=5, color_fp16=fp16, temporal_bias=bias, update_rule=rule) for _ in range(2))
+    b.set_pipeline(False)
+    if shape:
+        a.set_pipeline(True, *shape)
+    raw = _seeded_state(a, K, w * h, rng)
+    outs = [torch.zeros((h, w, 3), device="cuda") for _ in range(2)]
+    for st in (a, b):
+        st.import_raw(raw, 7)
+    odd = torch.tensor([float("inf"), -float("inf"), float("nan"), 1e6, -0.0, 3e38], device="cuda")
+    for t in range(18):
+        frame = torch.rand((h, w, 3), device="cuda", generator=gen)
+        at = torch.randint(0, frame.numel(), (200,), device="cuda", generator=gen)
+        frame.view(-1)[at] = odd[torch.randint(0, len(odd), (200,), device="cuda", generator=gen)]
+        fm = torch.where(torch.rand((h, w), device="cuda", generator=gen) < 0.2, 255, 3).to(torch.uint8) if t % 3 else None
+        for st, o in zip((a, b), outs):
+            st.push_frame(frame, (400.0 + 9 * t, 311.0), fov_map=fm, out=o)
+        assert torch.equal(outs[0].view(torch.int32), outs[1].view(torch.int32)), t
+    assert a.check_status() == 0 and b.check_status() == 0
+    assert np.array_equal(a.export_raw()[256:], b.export_raw()[256:])
+    assert a.replacements() == b.replacements()
