@@ -86,8 +86,8 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // per plane segment. The tile starts at pixel p0 (a multiple of T >= 256);
 // requires frame rows without padding and 16-byte aligned frame and state
 // planes. A bulk copy moves whole 16 bytes, four pixels of the frame: up to
-// three last pixels of an image come by plain loads. copy_frame = false leaves the frame segment to the
-// consumers (they foveate the frame into it themselves).
+// three last pixels of an image come by plain loads. copy_frame = false leaves
+// the frame segment to the warps that foveate the frame into it.
 // AHEAD: also bring what the tile's fold will read into the L2.
 template <int T, bool AHEAD>
 __device__ __forceinline__ void issue_tile_copies(const StreamDev& s, const FrameDev& f, int K,
@@ -363,8 +363,9 @@ constexpr int kMaxStages = 8;
 constexpr int kAnswers = kMaxStages + 2;
 
 // Shared-memory ring of S stages, each holding one tile's planes followed by
-// its uniforms and, if some frame has a flush map, its flush-map entries, then the S "full" and S "empty" barriers, and the answers of
-// the work queue with theirs.
+// its uniforms and, if some frame has a flush map, its flush-map entries; then
+// the answers of the work queue, the S "full" and S "empty" barriers, the
+// answers' barriers and a flag word.
 struct Ring {
   uint8_t* base;
   uint32_t stage_bytes;  // planes of the largest tile layout used
@@ -416,8 +417,9 @@ __device__ __forceinline__ Ring make_ring(uint8_t* smem, uint32_t stage_bytes, i
 }
 
 // One warp initialises the barriers (full: one arrival per producing warp, the
-// copying, the drawing and any foveating ones; empty: one arrival per consumer warp; told: the
-// request's) and the flag; the caller then synchronises the block.
+// copying, the drawing and any foveating ones; empty: one arrival per consumer
+// warp; told: the request's) and the flag; the caller then synchronises the
+// block.
 __device__ __forceinline__ void init_ring(const Ring& r, int consumer_warps, int producer_warps, int lane) {
   if (lane < r.S) {
     mbar_init(&r.full[lane], producer_warps);

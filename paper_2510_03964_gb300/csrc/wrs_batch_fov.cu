@@ -1,7 +1,7 @@
 // The foveating variants of the batched kernel (wrs_push_batch_foveated):
 // every stream's frame is foveated on read from its rendered image and mip
-// levels (Sec. 4.3's post-process) by the consumers, as wrs_push_foveated
-// does for one stream; instantiated here, apart from the plain batches, so the
+// levels (Sec. 4.3's post-process) by two warps of each CTA, as
+// wrs_push_foveated does for one stream; instantiated here, apart from the plain batches, so the
 // two sets compile in parallel.
 #include "wrs_batch_kernel.cuh"
 #include "wrs_internal.h"

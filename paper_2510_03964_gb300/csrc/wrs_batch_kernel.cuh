@@ -92,8 +92,9 @@ __device__ __forceinline__ int tile(const BatchEntry& e, uint8_t* st, const floa
   return wrs::compute_tile<KT, F16, PX, T, LIT>(e.s, e.f, st, u, px, d_f, tid);
 }
 
-// The copying warp's work for one tile of entry e. KT, CS > 0 fix the slot count and colour bytes at compile time (the
-// K = 4 / 8 families), so the copy sizes and stage offsets fold to constants.
+// The copying warp's work for one tile of entry e. KT, CS > 0 fix the slot
+// count and colour bytes at compile time (the K = 4 / 8 families), so the copy
+// sizes and stage offsets fold to constants.
 template <int T, int KT, int CS, bool COPY_FRAME>
 __device__ __forceinline__ void produce_tile(const BatchEntry& e, int64_t p0, uint8_t* st,
                                              uint64_t* full, int ln, uint32_t stage_cap,

@@ -607,13 +607,12 @@ __device__ __forceinline__ void fold_store(const StreamDev& s, uint32_t* idx, in
 // inputs were loaded ahead, else loaded here). KM >= K: the capacity of the
 // preloaded inputs (a batched kernel loads for up to 8 slots whatever the
 // stream's K; entries past K are dead code once K is a constant).
-// AHEAD: the caller has tested the band and loaded (pre) or not.
-template <int KT, int KM = FoldCap<KT>::value, bool AHEAD = false>
+template <int KT, int KM = FoldCap<KT>::value>
 __device__ __forceinline__ void record_code(const StreamDev& s, const FrameDev& f, int64_t p,
                                             uint8_t c, const FoldIn<KM>* pre) {
   const int K = KT > 0 ? KT : s.K;
   s.maps[static_cast<int64_t>(f.t & kRingMask) * s.plane + p] = c;
-  if (AHEAD ? pre == nullptr : !folds_now(f, p)) return;
+  if (!folds_now(f, p)) return;
   if (pre != nullptr) {
     fold_store(s, s.idx, K, f.t, f.map_lo, p, *pre, c);
   } else {
@@ -703,8 +702,7 @@ __device__ __forceinline__ int push_group(const StreamDev& s, const FrameDev& f,
 #pragma unroll
     for (int i = 0; i < PX; ++i) {
       if (valid[i]) {
-        const float* fp = src.frame ? src.frame + 3 * i
-                                    : f.frame + static_cast<int64_t>(ys[i]) * f.pitch + 3 * xs[i];
+        const float* fp = f.frame + static_cast<int64_t>(ys[i]) * f.pitch + 3 * xs[i];
         rgb[i][0] = fp[0]; rgb[i][1] = fp[1]; rgb[i][2] = fp[2];
       } else {
         rgb[i][0] = rgb[i][1] = rgb[i][2] = 0.0f;
@@ -920,8 +918,7 @@ __device__ __forceinline__ int push_group_literal(const StreamDev& s, const Fram
 #pragma unroll
     for (int i = 0; i < PX; ++i) {
       if (valid[i]) {
-        const float* fp = src.frame ? src.frame + 3 * i
-                                    : f.frame + static_cast<int64_t>(ys[i]) * f.pitch + 3 * xs[i];
+        const float* fp = f.frame + static_cast<int64_t>(ys[i]) * f.pitch + 3 * xs[i];
         rgb[i][0] = fp[0]; rgb[i][1] = fp[1]; rgb[i][2] = fp[2];
       } else {
         rgb[i][0] = rgb[i][1] = rgb[i][2] = 0.0f;

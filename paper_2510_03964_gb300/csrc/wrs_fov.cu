@@ -55,7 +55,6 @@ struct MipArgs {
   const float* img;
   int64_t pitch;
   int32_t width, height;
-  int32_t top;                          // highest level built, 1..WRS_MAX_MIP_LEVELS-1
   MipLevelOut lev[WRS_MAX_MIP_LEVELS];  // [0] unused
 };
 
@@ -305,7 +304,6 @@ extern "C" int wrs_mip_build(const float* d_img, int64_t pitch, int32_t width, i
   a.pitch = pitch;
   a.width = width;
   a.height = height;
-  a.top = levels - 1;
   fill_levels(L, d_mip, a.lev);
   const int M = levels - 1;
   const dim3 grid((unsigned)(((int64_t)width + kMipTileW - 1) / kMipTileW),
@@ -357,7 +355,6 @@ int wrs_fov_check_source(const float* d_img, int64_t pitch, const void* d_mip, s
                     nradii + 1, (long long)L.total_bytes);
   fv.img = d_img;
   fv.pitch = pitch;
-  fv.nradii = nradii;
   fill_levels(L, d_mip, fv.lev);
   *out = fv;
   return WRS_OK;
@@ -393,7 +390,7 @@ extern "C" int wrs_foveate(const float* d_img, int64_t pitch, const void* d_mip,
   const int64_t th = box ? FovTile<WRS_FILTER_BOX>::kH : FovTile<WRS_FILTER_BILINEAR>::kH;
   const int64_t want = quad ? ((width + tw - 1) / tw) * ((height + th - 1) / th)
                             : ((int64_t)width * height + kFovThreads - 1) / kFovThreads;
-  const int64_t cap = (int64_t)sms * 8 * 16;  // 8 resident CTAs per SM x 16 waves
+  const int64_t cap = (int64_t)sms * 128;  // about 25 waves of the five CTAs per SM
   const unsigned grid = (unsigned)(want < cap ? want : cap);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const auto kernel = quad ? (box ? foveate4_kernel<WRS_FILTER_BOX>

@@ -10,10 +10,10 @@
 
 namespace wrs {
 
-// Programmatic dependent launch: a kernel of this library (launch_early) starts on
-// the SMs that the previous kernel of the stream has left and sets up its
-// barriers there; grid_begin then waits until that kernel has completed and its writes
-// are visible. Nothing before grid_begin touches global memory, and every CTA
+// Programmatic dependent launch: a kernel of this library (wrs_launch_early)
+// starts on the SMs that the previous kernel of the stream has left and sets up
+// its barriers there; grid_begin then waits until that kernel has completed and
+// its writes are visible. Nothing before grid_begin touches global memory, and every CTA
 // calls it. A kernel that calls it reads with ordinary loads: what the previous
 // kernel writes changes while this one runs, and the compiler may move a
 // non-coherent load (__ldg) across the wait.
@@ -32,9 +32,8 @@ struct MipLevelDev {
 struct FovDev {
   const float* img;                     // [H][pitch] RGB triples
   int64_t pitch;
-  int32_t nradii;                       // 1..WRS_MAX_MIP_LEVELS-1
-  float r2[WRS_MAX_MIP_LEVELS - 1];     // r_i * r_i, rounded once; infinite past nradii
-  MipLevelDev lev[WRS_MAX_MIP_LEVELS];  // [1..nradii]; [0] unused (the image)
+  float r2[WRS_MAX_MIP_LEVELS - 1];     // r_i * r_i, rounded once; infinite past the last radius
+  MipLevelDev lev[WRS_MAX_MIP_LEVELS];  // one per radius from [1]; [0] unused (the image)
 };
 
 // Level coordinate of pixel index i at level L: u = (i + 0.5) * 2^-L - 0.5

@@ -154,8 +154,9 @@ uint32_t* wrs_status_word(const wrs_ctx* x) {
 }
 
 // Stages of `px` pixels per thread: as many (up to four) as keep two CTAs on
-// an SM, else what one CTA holds. More stages keep more bytes in flight; the
-// kernels wait on copies, not on arithmetic.
+// an SM, else what one CTA holds. More stages keep more bytes in flight, and a
+// second CTA the consumer warps that hide the arithmetic's latency (see
+// wrs_staged.cuh).
 int wrs_default_stages(int K, bool f16, int px) {
   constexpr size_t kSmPerSm = 228 * 1024, kReservedPerCta = 1024;
   int st = 4;
@@ -506,7 +507,7 @@ extern "C" int wrs_push_foveated(wrs_ctx* x, const float* d_img, int64_t img_pit
   if (x->t == 0xFFFFFFFFu) return wrs_fail(WRS_ERR_STATE, "frame counter exhausted");
   const StreamDev s = wrs_stream_dev(x);
   FrameDev f;
-  f.frame = nullptr;  // the consumers foveate the frame into shared memory
+  f.frame = nullptr;  // two warps of each CTA foveate the frame into shared memory
   f.pitch = 3 * static_cast<int64_t>(x->cfg.width);
   f.fov = d_fov;
   f.out = d_out;

@@ -1,9 +1,9 @@
 // Pipelined persistent form of the fused update + resolve (sm_103a).
 //
 // The CTAs that fit on the GPU take the image's tiles of T = 256 * PX pixels in
-// ascending order from the hardware's work queue (request_tile). A copying warp streams the planes a tile needs (frame
-// RGB, W, P, the K key planes and, for the fused resolve, the K slot records)
-// into a ring of S shared-memory stages with 1-D bulk asynchronous copies
+// ascending order from the hardware's work queue (request_tile). A copying warp
+// streams the planes a tile needs (frame RGB, W, P, the K key planes and, for
+// the fused resolve, the K slot records) into a ring of S shared-memory stages with 1-D bulk asynchronous copies
 // (cp.async.bulk) that complete on one transaction-count "full" mbarrier per
 // stage; a drawing warp adds the tile's uniforms (one Philox block per 4
 // pixels). With one warp doing both, the draw (about 220 dependent
@@ -49,8 +49,8 @@ constexpr int pipe_threads(int fovf) { return (kConsumerWarps + producers(fovf))
 // Resident CTAs per SM the compiler is asked to fit: three for one or two
 // slots and one pixel per thread and for the literal rule at up to two (their
 // stages are small, and the extra warps hide the per-pixel arithmetic's
-// latency: 4K literal rule, 24 against 16 consumer warps per SM, 68.7 -> 63.9 us), two for
-// one pixel per thread, else one.
+// latency: 4K literal rule, 24 against 16 consumer warps per SM, 68.7 -> 63.9
+// us), two for one pixel per thread, else one.
 template <int KT, int PX, bool LIT, int FOVF>
 constexpr int pipe_min_blocks() {
   if (FOVF >= 0) return 2;
@@ -191,7 +191,7 @@ cudaError_t plan_pipe_t(const StreamDev& s, const FrameDev& f, PipeArgs a, int s
 // any other through the generic instantiation, and the literal rule.
 template <bool F16, int FILTER>
 cudaError_t plan_pipe_fov_k(const StreamDev& s, const FrameDev& f, const FovDev& fv,
-                              const PipeArgs& a, int sms, int ctas, wrs_pipe_plan* plan) {
+                            const PipeArgs& a, int sms, int ctas, wrs_pipe_plan* plan) {
   if (s.literal) return plan_pipe_t<1, F16, 1, true, FILTER>(s, f, a, sms, ctas, plan, fv);
   switch (s.K) {
     case 4: return plan_pipe_t<4, F16, 1, false, FILTER>(s, f, a, sms, ctas, plan, fv);
@@ -204,7 +204,7 @@ cudaError_t plan_pipe_fov_k(const StreamDev& s, const FrameDev& f, const FovDev&
 
 template <int KT, bool F16, bool LIT = false>
 cudaError_t plan_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
-                            wrs_pipe_plan* plan) {
+                         wrs_pipe_plan* plan) {
   switch (px) {
     case 4: return plan_pipe_t<KT, F16, 4, LIT>(s, f, a, sms, ctas, plan);
     case 2: return plan_pipe_t<KT, F16, 2, LIT>(s, f, a, sms, ctas, plan);
@@ -214,7 +214,7 @@ cudaError_t plan_pipe_px(const StreamDev& s, const FrameDev& f, const PipeArgs& 
 
 template <bool F16>
 cudaError_t plan_pipe_k(const StreamDev& s, const FrameDev& f, const PipeArgs& a, int px, int sms, int ctas,
-                           wrs_pipe_plan* plan) {
+                        wrs_pipe_plan* plan) {
   if (s.literal) return plan_pipe_px<1, F16, true>(s, f, a, px, sms, ctas, plan);
   switch (s.K) {
     case 1: return plan_pipe_px<1, F16>(s, f, a, px, sms, ctas, plan);
@@ -248,8 +248,8 @@ bool wrs_pipe_supported(const wrs_ctx* x, const float* frame, int64_t pitch, con
 }
 
 cudaError_t wrs_plan_pipe_fov(const StreamDev& s, const FrameDev& f, const FovDev& fv, int filter,
-                                bool f16, int stages, int sms, int ctas_per_sm, uint32_t* status,
-                                uint64_t timeout_ns, uint32_t extra_tx, wrs_pipe_plan* plan) {
+                              bool f16, int stages, int sms, int ctas_per_sm, uint32_t* status,
+                              uint64_t timeout_ns, uint32_t extra_tx, wrs_pipe_plan* plan) {
   PipeArgs a;
   a.stages = stages;
   a.resolve = (f.out != nullptr || s.bias == 2) ? 1 : 0;  // records: resolve or Delta L
@@ -264,8 +264,8 @@ cudaError_t wrs_plan_pipe_fov(const StreamDev& s, const FrameDev& f, const FovDe
 }
 
 cudaError_t wrs_plan_pipe(const StreamDev& s, const FrameDev& f, bool f16, int px, int stages,
-                            int sms, int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
-                            uint32_t extra_tx, wrs_pipe_plan* plan) {
+                          int sms, int ctas_per_sm, uint32_t* status, uint64_t timeout_ns,
+                          uint32_t extra_tx, wrs_pipe_plan* plan) {
   PipeArgs a;
   a.stages = stages;
   a.resolve = (f.out != nullptr || s.bias == 2) ? 1 : 0;  // records: resolve or Delta L

@@ -2,10 +2,11 @@
 // consumer warps of the pipelined and the batched kernels run. The arithmetic
 // is push_group's (wrs_device.cuh), step for step and bit for bit.
 //
-// What bounds it: instruction issue and its latency. An SM holds 16 consumer
-// warps (shared memory allows no more pixels in flight), so each pixel's
-// instructions, not DRAM, set the time of every form that moves less than the
-// FP32 K = 8 one. Hence, against push_group:
+// What bounds it: instruction issue and its latency, with DRAM close behind.
+// An SM holds 16 consumer warps (shared memory allows no more pixels in flight),
+// so each pixel's instructions set the time of the forms that move little per
+// pixel (HD K = 4, the literal rule, flushes, the full bias); 4K K = 8 is at its
+// DRAM traffic. Hence, against push_group:
 //  * a thread owns its pixels' columns of the stage, so the rare events (a
 //    flush, a rescale of the keys, the replaced slot) are written into the
 //    columns and the loops over the slots then read them as they are: no
@@ -15,7 +16,8 @@
 // Measured against push_group on the same stages: 4K K = 8 FP16 286 -> 247 us,
 // 4K K = 8 FP32 295 -> 282 us (mostly DRAM), HD K = 4 FP32 55.5 -> 48.7 us, 4K
 // literal rule 82.8 -> 73.8 us; executed instructions per pixel 770 -> 610
-// (K = 8 FP16), 540 -> 450 (K = 4 FP32).
+// (K = 8 FP16), 540 -> 450 (K = 4 FP32), and 570 and 425 with the folds by
+// shifts and the flush maps in the stage.
 #pragma once
 
 #include <stdint.h>
