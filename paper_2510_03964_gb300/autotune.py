@@ -25,6 +25,7 @@ import threading
 import torch
 
 from . import build as _build
+from . import kernel_source_hash
 from ._lib import WrsError
 from .wrs import Batch, Stream
 
@@ -39,7 +40,7 @@ BATCH_CANDIDATES = [(px, st, ctas, g) for px in (1, 2) for st in (0, 2, 3) for c
 
 def _key(kind: str, shapes) -> str:
     name = torch.cuda.get_device_name()
-    return f"{name}|{_build.fingerprint()}|{kind}|" + ";".join(",".join(str(v) for v in s) for s in shapes)
+    return f"{name}|{kernel_source_hash()}|{kind}|" + ";".join(",".join(str(v) for v in s) for s in shapes)
 
 
 def _load_cache() -> dict:

@@ -13,7 +13,6 @@ from __future__ import annotations
 
 import concurrent.futures as cf
 import glob
-import hashlib
 import os
 import shutil
 import subprocess
@@ -52,14 +51,6 @@ def is_stale(lib: str = LIB) -> bool:
         return True
     t = os.path.getmtime(lib)
     return any(os.path.getmtime(d) > t for d in _deps())
-
-
-def fingerprint() -> str:
-    """Digest of the sources the libraries are built from."""
-    h = hashlib.sha256()
-    for d in _deps():
-        h.update(open(d, "rb").read())
-    return h.hexdigest()[:16]
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,

@@ -9,7 +9,9 @@
 // goes through the same bulk-copy / uniform / compute pipeline as the
 // single-stream kernel (wrs_async.cuh), with the arithmetic chosen per tile by
 // the stream's K and colour precision; results are bit-identical to pushing
-// each stream on its own.
+// each stream on its own. Batches of other slot counts, the literal rule or
+// mixed colours are pushed through each stream's own kernel where that is
+// faster (wrs_own.cu).
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -228,7 +228,7 @@ def test_a_tuned_launch_shape_belongs_to_the_sources_it_was_tuned_with(tmp_path,
     monkeypatch.setattr(torch.cuda, "get_device_name", lambda: "GB300")
     src = tmp_path / "kernel.cu"
     src.write_text("// one tile per CTA\n")
-    monkeypatch.setattr(build, "_deps", lambda: [str(src)])
+    monkeypatch.setattr(build, "CSRC", str(tmp_path))
     keys = [autotune._key("stream", [(64, 32, 4, 0)]), autotune._key("stream", [(64, 32, 4, 0)])]
     src.write_text("// a fixed deal\n")
     keys.append(autotune._key("stream", [(64, 32, 4, 0)]))
