@@ -294,8 +294,10 @@ __all__ = ["Stream", "make_config", "state_bytes", "state_layout", "unpack_state
 
 
 class Batch:
-    """One persistent launch (a CUDA-graph kernel node) that pushes a frame into
-    each of up to ``max_streams`` streams of any size, K and colour precision."""
+    """One launch that pushes a frame into each of up to ``max_streams`` streams
+    of any size, K and colour precision: a persistent kernel over all of them (a
+    CUDA-graph kernel node) or, for large streams of other slot counts than 4 and
+    8, a graph of the streams' own kernels."""
 
     def __init__(self, max_streams: int = 64):
         b = C.c_void_p()
